@@ -358,8 +358,9 @@ void mvd_batch_destroy(mvd_batch* batch);
  * the context's own data (the estimate is restored afterwards), then sets the
  * fastest on the context. Candidates: the FFT engine with register-resident
  * power-of-two passes and with mixed-radix Stockham passes (where the dims
- * are {2,3,5}-smooth), and the direct engine with output tiles of 32 x ty x 4
- * for every ty in {8,4,2,1} whose staging fits in shared memory.
+ * are {2,3,5}-smooth), and the direct engine with ty = 8 (output tiles of 16 or
+ * 8 rows, whichever its cost rule estimates cheaper) and ty = 4 (8 rows; 2 and
+ * 1, which an older cache may hold, mean the same).
  * The choice is persisted per (dims, precision, PSF boxes, GPU model) as one
  * text line appended to cache_path (NULL = the MVD_TUNE_CACHE environment
  * variable; neither = not persisted). An existing entry is applied without
@@ -370,7 +371,7 @@ void mvd_batch_destroy(mvd_batch* batch);
  */
 typedef struct {
     int path;             /* MVD_PATH_DIRECT or MVD_PATH_FFT */
-    int direct_tile_y;    /* direct engine: output tile height ty; 0 for FFT */
+    int direct_tile_y;    /* direct engine: output tile choice ty (see above); 0 for FFT */
     int fft_engine;       /* FFT: 1 register-resident passes, 0 Stockham passes; -1 for direct */
     int from_cache;       /* 1 when read from the cache without timing */
     double ms_per_update; /* measured time of one view update (ms) */

@@ -27,7 +27,7 @@
 #include <cmath>
 #include <vector>
 
-#include "box_sum.cuh"
+#include "box_conv.cuh"
 #include "common.cuh"
 #include "dd.cuh"
 
@@ -199,85 +199,13 @@ struct KBox {
     }
 };
 
-// One warp per output value (blocks of kThreads threads hold kThreads / 32
-// outputs); i = the output's index, uniform within the warp.
-__device__ __forceinline__ int warp_item() { return (int)((blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5); }
-inline int warp_blocks(long n) { return (int)((n * 32 + kThreads - 1) / kThreads); }
-
-// out(d) = sum_e a(e) g(d - e), d and e on box a
-__global__ void k_kconv(const float* a, KBox ba, const float* g, KBox bg, float* out) {
-    const int i = warp_item();
-    if (i >= ba.size()) return;
-    int dx, dy, dz;
-    ba.offset(i, dx, dy, dz);
-    const float s = warp_box_sum(max(-ba.hx(), dx - bg.hx()), min(ba.hx(), dx + bg.hx()),
-                                 max(-ba.hy(), dy - bg.hy()), min(ba.hy(), dy + bg.hy()),
-                                 max(-ba.hz(), dz - bg.hz()), min(ba.hz(), dz + bg.hz()),
-                                 [&](int ex, int ey, int ez, float acc) {
-                                     return fmaf(a[ba.index(ex, ey, ez)], g[bg.index(dx - ex, dy - ey, dz - ez)], acc);
-                                 });
-    if ((threadIdx.x & 31) == 0) out[i] = s;
-}
-
-// ab(e) += sum_d cb(d) g(d - e)   (adjoint of k_kconv in a), d and e on box a
-__global__ void k_kconv_ta(const float* cb, KBox ba, const float* g, KBox bg, float* ab) {
-    const int i = warp_item();
-    if (i >= ba.size()) return;
-    int ex, ey, ez;
-    ba.offset(i, ex, ey, ez);
-    const float s = warp_box_sum(max(-ba.hx(), ex - bg.hx()), min(ba.hx(), ex + bg.hx()),
-                                 max(-ba.hy(), ey - bg.hy()), min(ba.hy(), ey + bg.hy()),
-                                 max(-ba.hz(), ez - bg.hz()), min(ba.hz(), ez + bg.hz()),
-                                 [&](int dx, int dy, int dz, float acc) {
-                                     return fmaf(cb[ba.index(dx, dy, dz)], g[bg.index(dx - ex, dy - ey, dz - ez)], acc);
-                                 });
-    if ((threadIdx.x & 31) == 0) ab[i] += s;
-}
-
-// gb(f) = sum_e cb(e + f) a(e)   (adjoint of k_kconv in g), f on box g
-__global__ void k_kconv_tg(const float* cb, const float* a, KBox ba, float* gb, KBox bg) {
-    const int i = warp_item();
-    if (i >= bg.size()) return;
-    int fx, fy, fz;
-    bg.offset(i, fx, fy, fz);
-    const float s = warp_box_sum(max(-ba.hx(), -ba.hx() - fx), min(ba.hx(), ba.hx() - fx),
-                                 max(-ba.hy(), -ba.hy() - fy), min(ba.hy(), ba.hy() - fy),
-                                 max(-ba.hz(), -ba.hz() - fz), min(ba.hz(), ba.hz() - fz),
-                                 [&](int ex, int ey, int ez, float acc) {
-                                     return fmaf(cb[ba.index(ex + fx, ey + fy, ez + fz)], a[ba.index(ex, ey, ez)], acc);
-                                 });
-    if ((threadIdx.x & 31) == 0) gb[i] = s;
-}
-
-// Q(f) = sum_g P(g) P(g - f): pb(h) += sum_f qb(f) (P(h - f) + P(h + f)), h on box p,
-// f on box q (the two terms as two box sums: h - f in box p, h + f in box p)
-__global__ void k_autocorr_vjp(const float* qb, KBox bq, const float* p, KBox bp, float* pb) {
-    const int i = warp_item();
-    if (i >= bp.size()) return;
-    int hx, hy, hz;
-    bp.offset(i, hx, hy, hz);
-    const float s1 = warp_box_sum(max(-bq.hx(), hx - bp.hx()), min(bq.hx(), hx + bp.hx()),
-                                  max(-bq.hy(), hy - bp.hy()), min(bq.hy(), hy + bp.hy()),
-                                  max(-bq.hz(), hz - bp.hz()), min(bq.hz(), hz + bp.hz()),
-                                  [&](int fx, int fy, int fz, float acc) {
-                                      return fmaf(qb[bq.index(fx, fy, fz)], p[bp.index(hx - fx, hy - fy, hz - fz)], acc);
-                                  });
-    const float s2 = warp_box_sum(max(-bq.hx(), -bp.hx() - hx), min(bq.hx(), bp.hx() - hx),
-                                  max(-bq.hy(), -bp.hy() - hy), min(bq.hy(), bp.hy() - hy),
-                                  max(-bq.hz(), -bp.hz() - hz), min(bq.hz(), bp.hz() - hz),
-                                  [&](int fx, int fy, int fz, float acc) {
-                                      return fmaf(qb[bq.index(fx, fy, fz)], p[bp.index(hx + fx, hy + fy, hz + fz)], acc);
-                                  });
-    if ((threadIdx.x & 31) == 0) pb[i] += s1 + s2;
-}
-
-// pb(d) += ab(-d)
-__global__ void k_mirror_add(const float* ab, KBox b, float* pb) {
+// pb(d) += ab(-d) + sum_w ta_w(d): the gradient of A = P_v^* (ta_w: the factors' shares, already mirrored)
+__global__ void k_mirror_add(const float* ab, const float* ta, int nta, int n, float* pb) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= b.size()) return;
-    int dx, dy, dz;
-    b.offset(i, dx, dy, dz);
-    pb[i] += ab[b.index(-dx, -dy, -dz)];
+    if (i >= n) return;
+    float s = ab[n - 1 - i];
+    for (int w = 0; w < nta; ++w) s += ta[(size_t)w * n + i];
+    pb[i] += s;
 }
 
 // out(d) += vol(d mod dims) for d on the centred box b (a full correlation
@@ -402,105 +330,87 @@ mvd_status corr_to_box(const float* a, const float* b, const int dims[3], const 
 
 // scratch of the compound-kernel VJP, sized for the largest box
 struct VjpScratch {
-    float *A = nullptr, *U = nullptr, *Ab = nullptr, *Cb = nullptr, *Cf = nullptr, *Q = nullptr, *Gb = nullptr;
-    long qmax = 1;
+    float *A = nullptr, *U = nullptr, *Ab = nullptr, *Cb = nullptr, *Cf = nullptr, *Gb = nullptr;
     mvd_status alloc_for(const mvd_ctx* c) {
         long tmax = 1;
         for (int w = 0; w < c->nv; ++w) {
             const int* k = &c->kd[3 * w];
             tmax = std::max(tmax, (long)k[0] * k[1] * k[2]);
-            qmax = std::max(qmax, (long)(2 * k[0] - 1) * (2 * k[1] - 1) * (2 * k[2] - 1));
         }
         MVD_TRY(alloc(&A, tmax, "vjp A"));
         MVD_TRY(alloc(&U, tmax, "vjp U"));
         MVD_TRY(alloc(&Ab, tmax, "vjp Ab"));
         MVD_TRY(alloc(&Cb, (size_t)c->nv * tmax, "vjp Cb"));
         MVD_TRY(alloc(&Cf, (size_t)c->nv * tmax, "vjp C"));
-        MVD_TRY(alloc(&Q, (size_t)c->nv * qmax, "vjp Q"));
-        return alloc(&Gb, qmax, "vjp Gb");
+        return alloc(&Gb, (size_t)c->nv * c->qstride, "vjp Gb");
     }
     void release() {
-        for (float* p : {A, U, Ab, Cb, Cf, Q, Gb})
+        for (float* p : {A, U, Ab, Cb, Cf, Gb})
             if (p) cudaFree(p);
-        A = U = Ab = Cb = Cf = Q = Gb = nullptr;
+        A = U = Ab = Cb = Cf = Gb = nullptr;
     }
 };
 
-// compound-kernel VJP for view v: Pb[w] += d K_v / d Pn_w applied to Kb
+// compound-kernel VJP for view v: Pb[w] += d K_v / d Pn_w applied to Kb. With
+// A = P_v^*, G_w = Q_w (or P_w), C_w = A * G_w, each convolution a batch over w
+// (box_conv.cuh), written as sums over t of tap(t) in(d + t):
+//   C_w(d)   = sum_e A(e) G(d - e)    = sum_t P_v(t) G(d + t)
+//   Ab(-u)  += sum_d Cb(d) G(d + u)
+//   Gb(f)    = sum_e A(e) Cb(f + e)
+//   Pb_w(h) += sum_f Gb(f) (P(h - f) + P(h + f))
+//            = sum_t P(-t) Gb(h + t), and at -u sum_t P(t) Gb(u + t)
 static mvd_status compound_vjp(mvd_ctx* c, int v, const float* Kb, float* Pb, const VjpScratch& sc, cudaStream_t st) {
     const int nv = c->nv;
     const int* dv = &c->kd[3 * v];
     const int Tv = dv[0] * dv[1] * dv[2];
-    const KBox bv = kbox(dv);
     const float* Pv = c->d_psf + c->koff[v];
-    const long qmax = sc.qmax;
-    float *A = sc.A, *U = sc.U, *Ab = sc.Ab, *Cb = sc.Cb, *Cf = sc.Cf, *Q = sc.Q, *Gb = sc.Gb;
-    mvd_status stt = MVD_OK;
-    do {
-        if ((stt = mirror_kernel(Pv, dv, A, st)) != MVD_OK) break;
-        FactorPtrs fp{};
-        if (c->variant != MVD_PLAIN) {
-            for (int w = 0; w < nv && stt == MVD_OK; ++w) {
-                if (w == v) continue;
-                const int* dw = &c->kd[3 * w];
-                const float* Pw = c->d_psf + c->koff[w];
-                float* Cw = Cf + (size_t)w * Tv;
-                if (c->variant == MVD_EFFICIENT) {
-                    float* Qw = Q + (size_t)w * qmax;
-                    const int qd[3] = {2 * dw[0] - 1, 2 * dw[1] - 1, 2 * dw[2] - 1};
-                    if ((stt = autocorr_kernel(Pw, dw, Qw, st)) != MVD_OK) break;
-                    k_kconv<<<warp_blocks(Tv), kThreads, 0, st>>>(A, bv, Qw, kbox(qd), Cw);
-                } else if (c->variant == MVD_OPT1) {
-                    k_kconv<<<warp_blocks(Tv), kThreads, 0, st>>>(A, bv, Pw, kbox(dw), Cw);
-                } else {
-                    cudaError_t e = cudaMemcpyAsync(Cw, A, sizeof(float) * Tv, cudaMemcpyDeviceToDevice, st);
-                    if (e != cudaSuccess) {
-                        stt = cuda_status(e, "vjp factor copy");
-                        break;
-                    }
-                }
-                if (c->variant != MVD_OPT2) count_launch();
-                if ((stt = check_launch("vjp factor")) != MVD_OK) break;
-                fp.c[w] = Cw;
-            }
-            if (stt != MVD_OK) break;
+    float *A = sc.A, *U = sc.U, *Ab = sc.Ab, *Cb = sc.Cb, *Cf = sc.Cf;
+    const bool eff = c->variant == MVD_EFFICIENT, conv = eff || c->variant == MVD_OPT1;
+    MVD_TRY(mirror_kernel(Pv, dv, A, st));
+    FactorPtrs fp{};
+    std::vector<BoxJob> factors, ta, tg, back1, back2;
+    int slot = 0;
+    for (int w = 0; w < nv && c->variant != MVD_PLAIN; ++w) {
+        if (w == v) continue;
+        if (!conv) {  // OPT2: C_w = A
+            fp.c[w] = A;
+            continue;
         }
-        k_compound_back<<<1, 1024, 0, st>>>(A, fp, nv, Tv, Kb, U, Ab, Cb);
-        count_launch();
-        if ((stt = check_launch("vjp compound")) != MVD_OK) break;
-        for (int w = 0; w < nv && c->variant != MVD_PLAIN; ++w) {
-            if (w == v) continue;
-            const int* dw = &c->kd[3 * w];
-            const int Tw = dw[0] * dw[1] * dw[2];
-            const float* Pw = c->d_psf + c->koff[w];
-            float* Pbw = Pb + c->koff[w];
-            const float* Cbw = Cb + (size_t)w * Tv;
-            if (c->variant == MVD_OPT2) {  // C_w = A
-                k_add<<<blocks_for(Tv), kThreads, 0, st>>>(Ab, Cbw, Tv);
-                count_launch();
-                continue;
-            }
-            const int qd[3] = {2 * dw[0] - 1, 2 * dw[1] - 1, 2 * dw[2] - 1};
-            const float* G = c->variant == MVD_EFFICIENT ? Q + (size_t)w * qmax : Pw;
-            const KBox bg = c->variant == MVD_EFFICIENT ? kbox(qd) : kbox(dw);
-            k_kconv_ta<<<warp_blocks(Tv), kThreads, 0, st>>>(Cbw, bv, G, bg, Ab);
-            count_launch();
-            k_kconv_tg<<<warp_blocks(bg.kx * bg.ky * bg.kz), kThreads, 0, st>>>(Cbw, A, bv, Gb, bg);
-            count_launch();
-            if (c->variant == MVD_EFFICIENT) {
-                k_autocorr_vjp<<<warp_blocks(Tw), kThreads, 0, st>>>(Gb, bg, Pw, kbox(dw), Pbw);
-            } else {
-                k_add<<<blocks_for(Tw), kThreads, 0, st>>>(Pbw, Gb, Tw);
-            }
-            count_launch();
-            if ((stt = check_launch("vjp chain")) != MVD_OK) break;
+        const int* dw = &c->kd[3 * w];
+        const float* Pw = c->d_psf + c->koff[w];
+        const int gd[3] = {eff ? 2 * dw[0] - 1 : dw[0], eff ? 2 * dw[1] - 1 : dw[1], eff ? 2 * dw[2] - 1 : dw[2]};
+        const float* G = eff ? c->d_ktmp + (size_t)w * c->qstride : Pw;  // kept from the precompute
+        float* Cw = Cf + (size_t)slot * Tv;
+        const float* Cbw = Cb + (size_t)w * Tv;
+        float* Gb = sc.Gb + (size_t)w * c->qstride;
+        fp.c[w] = Cw;
+        factors.push_back(box_job(G, gd, Pv, dv, false, Cw, dv));
+        ta.push_back(box_job(G, gd, Cbw, dv, false, Cw, dv));  // the factors are read before
+        if (eff) {
+            tg.push_back(box_job(Cbw, dv, Pv, dv, true, Gb, gd));
+            back1.push_back(box_job(Gb, gd, Pw, dw, true, Pb + c->koff[w], dw, true));
+            back2.push_back(box_job(Gb, gd, Pw, dw, false, Pb + c->koff[w], dw, true, true));
+        } else {
+            tg.push_back(box_job(Cbw, dv, Pv, dv, true, Pb + c->koff[w], gd, true));
         }
-        if (stt != MVD_OK) break;
-        k_mirror_add<<<blocks_for(Tv), kThreads, 0, st>>>(Ab, bv, Pb + c->koff[v]);
+        ++slot;
+    }
+    MVD_TRY(box_convs(std::move(factors), st));
+    k_compound_back<<<1, 1024, 0, st>>>(A, fp, nv, Tv, Kb, U, Ab, Cb);
+    count_launch();
+    MVD_TRY(check_launch("vjp compound"));
+    MVD_TRY(box_convs(std::move(ta), st));
+    MVD_TRY(box_convs(std::move(tg), st));
+    MVD_TRY(box_convs(std::move(back1), st));
+    MVD_TRY(box_convs(std::move(back2), st));
+    for (int w = 0; w < nv && c->variant == MVD_OPT2; ++w) {
+        if (w == v) continue;
+        k_add<<<blocks_for(Tv), kThreads, 0, st>>>(Ab, Cb + (size_t)w * Tv, Tv);
         count_launch();
-        stt = check_launch("vjp mirror");
-    } while (false);
-    return stt;
+    }
+    k_mirror_add<<<blocks_for(Tv), kThreads, 0, st>>>(Ab, Cf, slot, Tv, Pb + c->koff[v]);
+    count_launch();
+    return check_launch("vjp mirror");
 }
 
 // Circular convolutions through the FP32 FFT engine: spectra of kernels or

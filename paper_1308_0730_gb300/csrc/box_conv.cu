@@ -1,0 +1,94 @@
+// Convolutions of small kernels with small kernels (the compound-kernel algebra
+// and its vector-Jacobian product), batched; tiling in box_conv.cuh.
+#include "box_conv.cuh"
+#include "common.cuh"
+
+namespace mvd {
+
+namespace {
+
+struct BoxJobs {
+    BoxJob j[kBcMaxJobs];
+};
+
+// two blocks per SM: the compensated sums take four registers per output
+template <int NY>
+__global__ void __launch_bounds__(256, 2) k_box_conv(const __grid_constant__ BoxJobs jobs, int splits) {
+    extern __shared__ float4 smem4[];
+    const BoxJob& b = jobs.j[blockIdx.y];
+    const int nz = 8 / splits;
+    const int tx = (b.c.ox + kBcTX - 1) / kBcTX, ty = (b.c.oy + 8 * NY - 1) / (8 * NY), tz = (b.c.oz + nz - 1) / nz;
+    const int t = blockIdx.x;
+    if (t >= tx * ty * tz) return;
+    bc_tile<NY, 0, false, true>(b.c, t % tx, (t / tx) % ty, t / (tx * ty), splits, reinterpret_cast<float*>(smem4),
+                             [&](int x, int y, int z, float acc) {
+        long g = (long)x + (long)b.c.ox * (y + (long)b.c.oy * z);
+        if (b.mirror) g = (long)b.c.ox * b.c.oy * b.c.oz - 1 - g;
+        b.out[g] = b.add ? b.out[g] + acc : acc;
+    });
+}
+
+}  // namespace
+
+mvd_status box_convs(std::vector<BoxJob> jobs, cudaStream_t st) {
+    for (size_t first = 0; first < jobs.size(); first += kBcMaxJobs) {
+        BoxJobs a{};
+        const int n = (int)(jobs.size() - first < (size_t)kBcMaxJobs ? jobs.size() - first : kBcMaxJobs);
+        long warps = 0;
+        int kz = 1;
+        for (int i = 0; i < n; ++i) {
+            const BoxConv& c = jobs[first + i].c;
+            a.j[i] = jobs[first + i];
+            warps += (long)((c.ox + 31) / 32) * ((c.oy + 7) / 8) * c.oz;
+            kz = c.kz > kz ? c.kz : kz;
+        }
+        // one tile height and split for the batch: the cheapest over all its boxes
+        int ny = 0, s = bc_splits(warps, kz);
+        BcPlan plan[kBcMaxJobs];
+        size_t smem = 0;
+        for (; ny == 0 && s <= 8; s *= 2) {
+            double best = 0.0;
+            for (int t = 2; t >= 1; t /= 2) {
+                double cost = 0.0;
+                size_t sm = 0;
+                BcPlan ps[kBcMaxJobs];
+                bool ok = true;
+                for (int i = 0; i < n && ok; ++i) {
+                    const BoxConv& c = a.j[i].c;
+                    BcPlan p{};
+                    ok = bc_plan_ny(c.ox, c.oy, c.oz, c.kx, c.ky, c.kz, t, s, 8, &p);
+                    cost += p.cost;
+                    sm = p.smem > sm ? p.smem : sm;
+                    ps[i] = p;
+                }
+                if (ok && (ny == 0 || cost < best)) {
+                    best = cost, ny = t, smem = sm;
+                    for (int i = 0; i < n; ++i) plan[i] = ps[i];
+                }
+            }
+            if (ny) break;
+        }
+        if (ny == 0) {
+            set_error("compound kernels: a PSF box is too large for the tiled convolution");
+            return MVD_ERR_UNSUPPORTED;
+        }
+        long tiles = 1;
+        const int nz = 8 / s;
+        for (int i = 0; i < n; ++i) {
+            BoxConv& c = a.j[i].c;
+            c.ck = plan[i].ck;
+            c.cy = plan[i].cy;
+            const long t = (long)((c.ox + 31) / 32) * ((c.oy + 8 * ny - 1) / (8 * ny)) * ((c.oz + nz - 1) / nz);
+            tiles = t > tiles ? t : tiles;
+        }
+        auto kern = ny == 2 ? k_box_conv<2> : k_box_conv<1>;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_status(e, "box convolutions");
+        kern<<<dim3((unsigned)tiles, (unsigned)n), 256, smem, st>>>(a, s);
+        count_launch();
+        MVD_TRY(check_launch("box convolutions"));
+    }
+    return MVD_OK;
+}
+
+}  // namespace mvd

@@ -152,14 +152,12 @@ mvd_status fft_inverse_real_fast(const FftGeom& g, const float2* S, float* dst, 
 
 // Direct (spatial) periodic convolution with fused epilogues.
 bool direct_supported(const int kd[3]);
-// ty = output tile height (8, 4, 2 or 1 rows of 32 x 4 outputs); 0 = the
-// largest whose staging fits in shared memory
+// ty = 0 or 8: the tile height the cost rule picks; 4, 2 or 1: eight rows per tile
 mvd_status direct_ratio(const int dims[3], const float* psi, const float* k, const int kd[3],
                         const float* phi, float eps, float* r, cudaStream_t st, int ty = 0);
 mvd_status direct_update(const int dims[3], const float* r, const float* k, const int kd[3],
                          float* psi, float eps, cudaStream_t st, int ty = 0, const float* wt = nullptr,
                          float lam = 0.f, const float* inv_s = nullptr);
-int direct_tile_heights(const int kd[3], int out[4]);  // tile heights that fit, largest first
 // prod *= r * k (the combined update's product of view factors)
 mvd_status direct_accumulate(const int dims[3], const float* r, const float* k, const int kd[3], float* prod,
                              cudaStream_t st, int ty = 0, const float* inv_s = nullptr);
@@ -167,15 +165,17 @@ mvd_status direct_conv(const int dims[3], const float* in, const float* k, const
                        float* out, cudaStream_t st);
 
 // Compound-kernel precompute and helpers.
-// compound kernel of view v into d_out; for MVD_EFFICIENT d_q holds Q_w = P_w * P_w^*
-// of every view w (autocorr_all) at stride qstride
-mvd_status build_compound(int n_views, const float* d_psf, const long* koff_h, const int* kd_h, int v,
-                          int variant, float* d_out, const float* d_q, long qstride, cudaStream_t st);
+// Q_w = P_w * P_w^* of every view w into d_q at stride qstride (box 2K - 1)
 mvd_status autocorr_all(int n_views, const float* d_psf, const long* koff_h, const int* kd_h, float* d_q,
                         long qstride, cudaStream_t st);
-mvd_status normalize_kernel(float* d_k, int n, int* d_bad, cudaStream_t st);
+// Compound kernels of every view, normalised to sum 1, into d_out (packed as d_psf); for
+// MVD_EFFICIENT d_q holds the autocorrelations. d_c: scratch for the factors P_v^* * G_w of
+// `group` views at a time, compound_scratch(...) floats. *d_bad is set where a sum is not > 0.
+size_t compound_scratch(int n_views, const int* kd_h, int variant, int* group);
+mvd_status build_compounds(int n_views, const float* d_psf, const long* koff_h, const int* kd_h, int variant,
+                           float* d_out, const float* d_q, long qstride, float* d_c, int group, int* d_bad,
+                           cudaStream_t st);
 mvd_status mirror_kernel(const float* k, const int kd[3], float* out, cudaStream_t st);
-mvd_status autocorr_kernel(const float* P, const int kd[3], float* Q, cudaStream_t st);  // Q box = 2K-1
 mvd_status direct_conv_add(const int dims[3], const float* in, const float* k, const int kd[3], float* out,
                            cudaStream_t st);
 mvd_status one_update(mvd_ctx* c, int v);
@@ -229,7 +229,8 @@ struct mvd_ctx {
     float* d_r = nullptr;      // M (direct-path ratio; scratch for kernel placement)
     float* d_psf = nullptr;    // packed normalised PSFs
     float* d_comp = nullptr;   // packed compound kernels
-    float* d_ktmp = nullptr;   // precompute scratch
+    float* d_ktmp = nullptr;   // precompute scratch; MVD_EFFICIENT: Q_w = P_w * P_w^* at w * qstride
+    long qstride = 0;
     double* d_red = nullptr;   // reduction scratch
     int* d_flag = nullptr;
 

@@ -4,10 +4,9 @@
 //   update: psi = max(psi . (r * K), eps)         (Eq. 15 / Eq. 220, second half)
 // (f * k)(x) = sum_d k(d) f((x - d) mod dims), d = tap index - (K-1)/2.
 //
-// Each block computes a TX x TY x TZ output tile. The input tile plus the
-// kernel's halo (periodically wrapped) and the kernel taps are staged in
-// shared memory; every thread accumulates TZ outputs along z, so each input
-// value it loads feeds up to TZ FMAs.
+// The tiling and its cost are in box_conv.cuh; the elementwise steps run in its
+// epilogue. Measured (GB300): see k_direct.
+#include "box_conv.cuh"
 #include "common.cuh"
 #include "fft.cuh"
 
@@ -15,161 +14,119 @@ namespace mvd {
 
 namespace {
 
-constexpr int TX = 32, TZ = 4;
+// The boxes this engine takes: those whose input tile (32 x 1 x 4 outputs plus
+// the box's halo) and taps fit in 200 KB of shared memory.
 constexpr size_t kMaxSmem = 200 * 1024;
 
-// tile height TY (8, 4, 2 or 1 rows of 32 threads): the largest whose input
-// tile + halo and kernel taps fit in shared memory
-inline size_t smem_bytes(const int kd[3], int ty) {
+inline bool box_fits(const int kd[3], int ty) {
     const size_t T = (size_t)kd[0] * kd[1] * kd[2];
-    const size_t tile = (size_t)(TX + kd[0] - 1) * (ty + kd[1] - 1) * (TZ + kd[2] - 1);
-    return (T + tile) * sizeof(float);
-}
-inline int pick_ty(const int kd[3]) {
-    for (int ty : {8, 4, 2, 1})
-        if (smem_bytes(kd, ty) <= kMaxSmem) return ty;
-    return 0;
+    const size_t tile = (size_t)(32 + kd[0] - 1) * (ty + kd[1] - 1) * (4 + kd[2] - 1);
+    return (T + tile) * sizeof(float) <= kMaxSmem;
 }
 
 struct DArgs {
-    int X, Y, Z, Kx, Ky, Kz;
-    const float* in;
-    const float* k;
+    BoxConv c;
     const float* phi;
     float* out;  // r (ratio), psi (update) or plain output
     float eps;
-    const float* wt;  // update: when set, apply the fraction wt of the change (partial overlap)
-    float lam;        // update: Tikhonov regularisation (0 = none)
+    const float* wt;     // update: when set, apply the fraction wt of the change (partial overlap)
+    float lam;           // update: Tikhonov regularisation (0 = none)
     const float* inv_s;  // update / accumulate: zero boundary, 1 / sensitivity
+    int splits, mode;
 };
 
-// MODE 0: out = phi / max(conv, eps); MODE 1: out = max(out . conv, eps); MODE 2: out = conv;
-// MODE 3: out += conv; MODE 4: out *= conv (the combined update's product)
-template <int MODE, int TY>
-__global__ void __launch_bounds__(TX * TY) k_direct(DArgs a) {
-    extern __shared__ float smem[];
-    const int T = a.Kx * a.Ky * a.Kz;
-    float* sk = smem;
-    float* st = smem + T;
-    const int WX = TX + a.Kx - 1, WY = TY + a.Ky - 1, WZ = TZ + a.Kz - 1;
-    const int hx = (a.Kx - 1) / 2, hy = (a.Ky - 1) / 2, hz = (a.Kz - 1) / 2;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * TZ;
+enum { M_RATIO, M_UPDATE, M_CONV, M_ADD, M_ACCUMULATE };
 
-    for (int i = threadIdx.x; i < T; i += blockDim.x) sk[i] = __ldg(a.k + i);
-    const int nt = WX * WY * WZ;
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-        const int ix = i % WX, r = i / WX, iy = r % WY, iz = r / WY;
-        int gx = (x0 - hx + ix) % a.X;
-        if (gx < 0) gx += a.X;
-        int gy = (y0 - hy + iy) % a.Y;
-        if (gy < 0) gy += a.Y;
-        int gz = (z0 - hz + iz) % a.Z;
-        if (gz < 0) gz += a.Z;
-        st[i] = __ldg(a.in + (long)gx + (long)a.X * (gy + (long)a.Y * gz));
-    }
-    __syncthreads();
-
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;  // ty < TY
-    float acc[TZ];
-#pragma unroll
-    for (int o = 0; o < TZ; ++o) acc[o] = 0.f;
-    // output o at tile z index o uses input plane i = o + (Kz-1) - kz
-    for (int ky = 0; ky < a.Ky; ++ky) {
-        const int iy = ty + (a.Ky - 1) - ky;
-        for (int kx = 0; kx < a.Kx; ++kx) {
-            const int ix = tx + (a.Kx - 1) - kx;
-            const float* col = st + ix + WX * iy;
-            const float* kcol = sk + kx + a.Kx * ky;
-            for (int i = 0; i < WZ; ++i) {
-                const float v = col[(long)WX * WY * i];
-#pragma unroll
-                for (int o = 0; o < TZ; ++o) {
-                    const int kz = o + (a.Kz - 1) - i;
-                    if (kz >= 0 && kz < a.Kz) acc[o] = fmaf(kcol[a.Kx * a.Ky * kz], v, acc[o]);
-                }
-            }
-        }
-    }
-    const int gx = x0 + tx, gy = y0 + ty;
-    if (gx >= a.X || gy >= a.Y) return;
-#pragma unroll
-    for (int o = 0; o < TZ; ++o) {
-        const int gz = z0 + o;
-        if (gz >= a.Z) break;
-        const long g = (long)gx + (long)a.X * (gy + (long)a.Y * gz);
-        if (MODE == 0)
-            a.out[g] = __ldg(a.phi + g) / fmaxf(acc[o], a.eps);
-        else if (MODE == 1)
-        {
+// M_RATIO: out = phi / max(conv, eps); M_UPDATE: out = max(out . conv, eps); M_CONV: out = conv;
+// M_ADD: out += conv; M_ACCUMULATE: out *= conv (the combined update's product). KX: the box's
+// length in x, 0 for those without a kernel of their own.
+template <int NY, int KX>
+__global__ void __launch_bounds__(NY == 1 ? 512 : 256, NY == 1 ? 1 : 3) k_direct(const __grid_constant__ DArgs a) {
+    extern __shared__ float4 smem4[];
+    bc_tile<NY, KX, true, false>(a.c, blockIdx.x, blockIdx.y, blockIdx.z, a.splits, reinterpret_cast<float*>(smem4),
+                                 [&](int x, int y, int z, float acc) {
+        const long g = (long)x + (long)a.c.ox * (y + (long)a.c.oy * z);
+        if (a.mode == M_RATIO) {
+            a.out[g] = __ldg(a.phi + g) / fmaxf(acc, a.eps);
+        } else if (a.mode == M_UPDATE) {
             const float p = a.out[g];
-            a.out[g] = fmaxf(p * (a.wt || a.lam != 0.f || a.inv_s ? update_factor(acc[o] - 1.f, p, a.wt, g, a.lam,
-                                                                                    a.inv_s)
-                                                                   : acc[o]),
+            a.out[g] = fmaxf(p * (a.wt || a.lam != 0.f || a.inv_s ? update_factor(acc - 1.f, p, a.wt, g, a.lam, a.inv_s)
+                                                                  : acc),
                              a.eps);
+        } else if (a.mode == M_CONV) {
+            a.out[g] = acc;
+        } else if (a.mode == M_ADD) {
+            a.out[g] += acc;
+        } else {
+            a.out[g] *= a.inv_s ? acc * __ldg(a.inv_s + g) : acc;
         }
-        else if (MODE == 2)
-            a.out[g] = acc[o];
-        else if (MODE == 3)
-            a.out[g] += acc[o];
-        else  // MODE 4: combined update, multiply this view's factor into the product
-            a.out[g] *= a.inv_s ? acc[o] * __ldg(a.inv_s + g) : acc[o];
+    });
+}
+
+template <int NY>
+auto kernel_for(int kx) {
+    switch (kx) {  // the short rows, whose loop and remainder would cost as much as their taps
+        case 3: return k_direct<NY, 3>;
+        case 5: return k_direct<NY, 5>;
+        case 7: return k_direct<NY, 7>;
+        case 9: return k_direct<NY, 9>;
+        case 11: return k_direct<NY, 11>;
+        case 13: return k_direct<NY, 13>;
+        case 15: return k_direct<NY, 15>;
+        case 17: return k_direct<NY, 17>;
+        default: return k_direct<NY, 0>;
     }
 }
 
-template <int MODE, int TY>
-mvd_status launch_ty(const DArgs& a, size_t sm, cudaStream_t st, const char* name) {
-    cudaError_t e = cudaFuncSetAttribute(k_direct<MODE, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+// ty 0 or 8: the cheaper of the 16- and 8-row tiles (bc_plan); 4, 2, 1: the 8-row tile
+mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty = 0) {
+    BoxConv& c = a.c;
+    const int kd[3] = {c.kx, c.ky, c.kz};
+    BcPlan p{};
+    if (!direct_supported(kd) || !bc_plan(c.ox, c.oy, c.oz, c.kx, c.ky, c.kz, ty == 0 || ty == 8 ? 2 : 1, &p)) {
+        set_error("%s: kernel box %dx%dx%d too large for the direct engine", name, kd[0], kd[1], kd[2]);
+        return MVD_ERR_UNSUPPORTED;
+    }
+    c.ck = p.ck;
+    c.cy = p.cy;
+    a.splits = p.s;
+    a.mode = mode;
+    auto kern = p.ny == 2 ? kernel_for<2>(c.kx) : kernel_for<1>(c.kx);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return cuda_status(e, name);
-    dim3 grid((a.X + TX - 1) / TX, (a.Y + TY - 1) / TY, (a.Z + TZ - 1) / TZ);
-    const int cls = MODE == 0 ? KC_DIRECT_RATIO : (MODE == 1 || MODE == 4) ? KC_DIRECT_UPDATE : KC_DIRECT_CONV;
+    const int nz = p.planes();
+    const dim3 grid((c.ox + kBcTX - 1) / kBcTX, (c.oy + 8 * p.ny - 1) / (8 * p.ny), (c.oz + nz - 1) / nz);
+    const int cls = mode == M_RATIO ? KC_DIRECT_RATIO
+                                    : (mode == M_UPDATE || mode == M_ACCUMULATE) ? KC_DIRECT_UPDATE : KC_DIRECT_CONV;
     prof_begin(cls, st);
-    k_direct<MODE, TY><<<grid, TX * TY, sm, st>>>(a);
+    kern<<<grid, 32 * p.warps, p.smem, st>>>(a);
     prof_end(cls, st);
     count_launch();
     return check_launch(name);
 }
 
-template <int MODE>
-mvd_status launch(const DArgs& a, const int kd[3], cudaStream_t st, const char* name, int ty_req = 0) {
-    const int ty = (ty_req == 8 || ty_req == 4 || ty_req == 2 || ty_req == 1) && smem_bytes(kd, ty_req) <= kMaxSmem
-                       ? ty_req
-                       : pick_ty(kd);
-    if (ty == 0) {
-        set_error("%s: kernel box %dx%dx%d too large for the direct engine", name, kd[0], kd[1], kd[2]);
-        return MVD_ERR_UNSUPPORTED;
-    }
-    const size_t sm = smem_bytes(kd, ty);
-    switch (ty) {
-        case 8: return launch_ty<MODE, 8>(a, sm, st, name);
-        case 4: return launch_ty<MODE, 4>(a, sm, st, name);
-        case 2: return launch_ty<MODE, 2>(a, sm, st, name);
-        default: return launch_ty<MODE, 1>(a, sm, st, name);
-    }
-}
-
+// (f * k)(x) = sum_t k(K - 1 - t) f(x + t - h): the taps reversed, the input starting h before the output
 DArgs make(const int dims[3], const float* in, const float* k, const int kd[3]) {
     DArgs a{};
-    a.X = dims[0];
-    a.Y = dims[1];
-    a.Z = dims[2];
-    a.Kx = kd[0];
-    a.Ky = kd[1];
-    a.Kz = kd[2];
-    a.in = in;
-    a.k = k;
+    BoxConv& c = a.c;
+    c.in = in;
+    c.taps = k;
+    c.ix = c.ox = dims[0];
+    c.iy = c.oy = dims[1];
+    c.iz = c.oz = dims[2];
+    c.kx = kd[0];
+    c.ky = kd[1];
+    c.kz = kd[2];
+    c.offx = -((kd[0] - 1) / 2);
+    c.offy = -((kd[1] - 1) / 2);
+    c.offz = -((kd[2] - 1) / 2);
+    c.mir = 1;
     return a;
 }
 
 }  // namespace
 
-bool direct_supported(const int kd[3]) { return pick_ty(kd) > 0; }
-
-int direct_tile_heights(const int kd[3], int out[4]) {
-    int n = 0;
-    for (int ty : {8, 4, 2, 1})
-        if (smem_bytes(kd, ty) <= kMaxSmem) out[n++] = ty;
-    return n;
-}
+bool direct_supported(const int kd[3]) { return box_fits(kd, 1); }
 
 mvd_status direct_ratio(const int dims[3], const float* psi, const float* k, const int kd[3],
                         const float* phi, float eps, float* r, cudaStream_t st, int ty) {
@@ -177,7 +134,7 @@ mvd_status direct_ratio(const int dims[3], const float* psi, const float* k, con
     a.phi = phi;
     a.out = r;
     a.eps = eps;
-    return launch<0>(a, kd, st, "direct ratio", ty);
+    return launch(a, M_RATIO, st, "direct ratio", ty);
 }
 
 mvd_status direct_update(const int dims[3], const float* r, const float* k, const int kd[3],
@@ -189,7 +146,7 @@ mvd_status direct_update(const int dims[3], const float* r, const float* k, cons
     a.wt = wt;
     a.lam = lam;
     a.inv_s = inv_s;
-    return launch<1>(a, kd, st, "direct update", ty);
+    return launch(a, M_UPDATE, st, "direct update", ty);
 }
 
 mvd_status direct_accumulate(const int dims[3], const float* r, const float* k, const int kd[3], float* prod,
@@ -197,21 +154,21 @@ mvd_status direct_accumulate(const int dims[3], const float* r, const float* k, 
     DArgs a = make(dims, r, k, kd);
     a.out = prod;
     a.inv_s = inv_s;
-    return launch<4>(a, kd, st, "direct accumulate", ty);
+    return launch(a, M_ACCUMULATE, st, "direct accumulate", ty);
 }
 
 mvd_status direct_conv(const int dims[3], const float* in, const float* k, const int kd[3], float* out,
                        cudaStream_t st) {
     DArgs a = make(dims, in, k, kd);
     a.out = out;
-    return launch<2>(a, kd, st, "direct conv");
+    return launch(a, M_CONV, st, "direct conv");
 }
 
 mvd_status direct_conv_add(const int dims[3], const float* in, const float* k, const int kd[3], float* out,
                            cudaStream_t st) {
     DArgs a = make(dims, in, k, kd);
     a.out = out;
-    return launch<3>(a, kd, st, "direct conv add");
+    return launch(a, M_ADD, st, "direct conv add");
 }
 
 }  // namespace mvd

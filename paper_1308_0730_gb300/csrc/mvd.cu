@@ -978,17 +978,15 @@ mvd_status mvd_precompute_kernels(mvd_ctx* c, int variant) {
         const int* k = &c->kd[3 * v];
         qmax = std::max(qmax, (size_t)(2 * k[0] - 1) * (2 * k[1] - 1) * (2 * k[2] - 1));
     }
-    MVD_TRY(dev_alloc(&c->d_ktmp, qmax * (size_t)c->nv, "precompute scratch"));
+    int group = 1;
+    const size_t nq = qmax * (size_t)c->nv, nc = compound_scratch(c->nv, c->kd.data(), variant, &group);
+    MVD_TRY(dev_alloc(&c->d_ktmp, nq + nc, "precompute scratch"));
+    c->qstride = (long)qmax;
     if (variant == MVD_EFFICIENT)
         MVD_TRY(autocorr_all(c->nv, c->d_psf, c->koff.data(), c->kd.data(), c->d_ktmp, (long)qmax, c->stream));
     MVD_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), c->stream));
-    for (int v = 0; v < c->nv; ++v) {
-        float* dst = c->d_comp + c->koff[v];
-        MVD_TRY(build_compound(c->nv, c->d_psf, c->koff.data(), c->kd.data(), v, variant, dst, c->d_ktmp,
-                               (long)qmax, c->stream));
-        const int* k = &c->kd[3 * v];
-        MVD_TRY(normalize_kernel(dst, k[0] * k[1] * k[2], c->d_flag, c->stream));
-    }
+    MVD_TRY(build_compounds(c->nv, c->d_psf, c->koff.data(), c->kd.data(), variant, c->d_comp, c->d_ktmp, (long)qmax,
+                            c->d_ktmp + nq, group, c->d_flag, c->stream));
     int bad = 0;
     MVD_TRY(read_flag(c, &bad));
     if (bad) {
@@ -1427,17 +1425,8 @@ mvd_status mvd_autotune(mvd_ctx* c, const char* cache_path, mvd_tune_result* out
             cands.push_back({MVD_PATH_FFT, 0, 0, 0.0});
         }
         if (direct_ok) {
-            // tile heights that fit every view's box
-            int common[4] = {8, 4, 2, 1};
-            for (int ty : common) {
-                bool fits = true;
-                for (int v = 0; v < c->nv; ++v) {
-                    int opts[4];
-                    const int n = direct_tile_heights(&c->kd[3 * v], opts);
-                    fits = fits && std::find(opts, opts + n, ty) != opts + n;
-                }
-                if (fits) cands.push_back({MVD_PATH_DIRECT, ty, 1, 0.0});
-            }
+            // the tile height of the cost rule, and the lowest
+            for (int ty : {8, 4}) cands.push_back({MVD_PATH_DIRECT, ty, 1, 0.0});
         }
         const int prev_path = c->path, prev_ty = c->direct_ty, prev_fast = c->geom.fast ? 1 : 0;
         for (size_t i = 0; i < cands.size() && st == MVD_OK; ++i) {

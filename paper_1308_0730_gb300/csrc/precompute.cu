@@ -6,7 +6,9 @@
 // (P_v^* * P_w * P_w^*) is linear convolution of those small functions. The
 // compound kernel of view v is zero outside P_v^*'s box, so every factor is
 // evaluated on that box only.
-#include "box_sum.cuh"
+#include <utility>
+
+#include "box_conv.cuh"
 #include "common.cuh"
 
 namespace mvd {
@@ -34,22 +36,6 @@ __device__ __forceinline__ void offset_of(const Box& b, int i, int& dx, int& dy,
     dz = r / b.ky - b.hz();
 }
 
-// Q(d) = sum_e P(e) P(e - d)   (P * P^*), on the box of size 2K-1; one warp per d
-__global__ void k_autocorr(const float* P, Box b, float* Q, Box q) {
-    const int i = (int)((blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5);
-    if (i >= q.size()) return;
-    int dx, dy, dz;
-    offset_of(q, i, dx, dy, dz);
-    // e and e - d both inside b
-    const int zlo = max(-b.hz(), dz - b.hz()), zhi = min(b.hz(), dz + b.hz());
-    const int ylo = max(-b.hy(), dy - b.hy()), yhi = min(b.hy(), dy + b.hy());
-    const int xlo = max(-b.hx(), dx - b.hx()), xhi = min(b.hx(), dx + b.hx());
-    const float s = warp_box_sum(xlo, xhi, ylo, yhi, zlo, zhi, [&](int ex, int ey, int ez, float acc) {
-        return fmaf(b.at(P, ex, ey, ez), b.at(P, ex - dx, ey - dy, ez - dz), acc);
-    });
-    if ((threadIdx.x & 31) == 0) Q[i] = s;
-}
-
 // out(d) = P^*(d) = P(-d)
 __global__ void k_mirror(const float* P, Box b, float* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -59,35 +45,32 @@ __global__ void k_mirror(const float* P, Box b, float* out) {
     out[i] = b.at(P, -dx, -dy, -dz);
 }
 
-// out(d) *= sum_e P^*(e) G(d - e)  for d on P's box  (P^*(e) = P(-e)); one warp per d
-__global__ void k_mul_conv(const float* P, Box b, const float* G, Box g, float* out) {
-    const int i = (int)((blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5);
-    if (i >= b.size()) return;
-    int dx, dy, dz;
-    offset_of(b, i, dx, dy, dz);
-    const int zlo = max(-b.hz(), dz - g.hz()), zhi = min(b.hz(), dz + g.hz());
-    const int ylo = max(-b.hy(), dy - g.hy()), yhi = min(b.hy(), dy + g.hy());
-    const int xlo = max(-b.hx(), dx - g.hx()), xhi = min(b.hx(), dx + g.hx());
-    const float s = warp_box_sum(xlo, xhi, ylo, yhi, zlo, zhi, [&](int ex, int ey, int ez, float acc) {
-        return fmaf(b.at(P, -ex, -ey, -ez), g.at(G, dx - ex, dy - ey, dz - ez), acc);
-    });
-    if ((threadIdx.x & 31) == 0) out[i] *= s;
-}
+// The compound kernels of up to kFinishViews views, one block each:
+// out = P^*(d) . prod_{w != v} C_w(d) (OPT2: C_w = P^*), then out /= sum(out) (the
+// sum in FP64); flag if the sum is not > 0.
+constexpr int kFinishViews = 32;
+struct Finish {
+    const float* p;  // P_v
+    const float* c;  // the first factor; factor i at c + i * size
+    float* out;
+    Box b;
+};
+struct FinishArgs {
+    Finish v[kFinishViews];
+};
 
-// out(d) *= P^*(d)
-__global__ void k_mul_mirror(const float* P, Box b, float* out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= b.size()) return;
-    int dx, dy, dz;
-    offset_of(b, i, dx, dy, dz);
-    out[i] *= b.at(P, -dx, -dy, -dz);
-}
-
-// one block: out /= sum(out) (sum in FP64); flag if the sum is not > 0
-__global__ void k_normalize(float* out, int n, int* bad) {
+__global__ void __launch_bounds__(1024) k_compound_finish(const __grid_constant__ FinishArgs a, int factors, int* bad) {
     __shared__ double part[1024];
+    const Finish& f = a.v[blockIdx.x];
+    const int n = f.b.size();
     double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += out[i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float m = __ldg(f.p + n - 1 - i);  // P(-d)
+        float u = m;
+        for (int w = 0; w < factors; ++w) u *= f.c ? f.c[(size_t)w * n + i] : m;
+        f.out[i] = u;
+        s += u;
+    }
     part[threadIdx.x] = s;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -100,7 +83,7 @@ __global__ void k_normalize(float* out, int n, int* bad) {
         return;
     }
     const float inv = (float)(1.0 / tot);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] *= inv;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) f.out[i] *= inv;
 }
 
 __global__ void k_place(const float* k, Box b, int X, int Y, int Z, float* vol) {
@@ -225,7 +208,6 @@ __global__ void k_fill(float* p, long n, float v) {
 
 inline Box box_of(const int* kd) { return Box{kd[0], kd[1], kd[2]}; }
 inline int blocks_for(long n) { return (int)((n + kThreads - 1) / kThreads); }
-inline int warp_blocks_for(long n) { return (int)((n * 32 + kThreads - 1) / kThreads); }  // one warp per output
 inline int grid_stride_blocks(long n) {
     long b = (n + kThreads - 1) / kThreads;
     return (int)(b < 152 * 8 ? (b < 1 ? 1 : b) : 152 * 8);
@@ -235,31 +217,61 @@ inline int grid_stride_blocks(long n) {
 
 mvd_status autocorr_all(int n_views, const float* d_psf, const long* koff, const int* kd, float* d_q, long qstride,
                         cudaStream_t st) {
-    for (int w = 0; w < n_views; ++w) MVD_TRY(autocorr_kernel(d_psf + koff[w], kd + 3 * w, d_q + (size_t)w * qstride, st));
-    return MVD_OK;
+    std::vector<BoxJob> jobs;  // Q(d) = sum_t P(t) P(d + t)
+    for (int w = 0; w < n_views; ++w) {
+        const int* k = kd + 3 * w;
+        const int q[3] = {2 * k[0] - 1, 2 * k[1] - 1, 2 * k[2] - 1};
+        jobs.push_back(box_job(d_psf + koff[w], k, d_psf + koff[w], k, false, d_q + (size_t)w * qstride, q));
+    }
+    return box_convs(std::move(jobs), st);
 }
 
-mvd_status build_compound(int n_views, const float* d_psf, const long* koff, const int* kd, int v,
-                          int variant, float* d_out, const float* d_q, long qstride, cudaStream_t st) {
-    const Box bv = box_of(kd + 3 * v);
-    const float* Pv = d_psf + koff[v];
-    k_mirror<<<blocks_for(bv.kx * bv.ky * bv.kz), kThreads, 0, st>>>(Pv, bv, d_out);
-    count_launch();
-    MVD_TRY(check_launch("compound mirror"));
-    if (variant != MVD_PLAIN) {
-        for (int w = 0; w < n_views; ++w) {
-            if (w == v) continue;
-            const Box bw = box_of(kd + 3 * w);
-            const float* Pw = d_psf + koff[w];
-            if (variant == MVD_EFFICIENT) {  // Q_w = P_w * P_w^*, computed once per view by autocorr_all
-                const Box bq{2 * bw.kx - 1, 2 * bw.ky - 1, 2 * bw.kz - 1};
-                k_mul_conv<<<warp_blocks_for(bv.kx * bv.ky * bv.kz), kThreads, 0, st>>>(Pv, bv, d_q + (size_t)w * qstride,
-                                                                                        bq, d_out);
-            } else if (variant == MVD_OPT1) {
-                k_mul_conv<<<warp_blocks_for(bv.kx * bv.ky * bv.kz), kThreads, 0, st>>>(Pv, bv, Pw, bw, d_out);
-            } else {
-                k_mul_mirror<<<blocks_for(bv.kx * bv.ky * bv.kz), kThreads, 0, st>>>(Pv, bv, d_out);
+// views whose factors are held at once: as many as keep the scratch below 64 MB,
+// at least one (more pairs per launch fill the last wave of tiles better)
+size_t compound_scratch(int n_views, const int* kd, int variant, int* group) {
+    *group = n_views;
+    if ((variant != MVD_EFFICIENT && variant != MVD_OPT1) || n_views < 2) return 0;
+    size_t most = 1;
+    for (int v = 0; v < n_views; ++v) {
+        const size_t t = (size_t)kd[3 * v] * kd[3 * v + 1] * kd[3 * v + 2];
+        most = t > most ? t : most;
+    }
+    const size_t per_view = most * (n_views - 1), cap = (size_t)16 << 20;
+    const size_t g = cap / per_view;
+    *group = g < 1 ? 1 : (g < (size_t)n_views ? (int)g : n_views);
+    return per_view * *group;
+}
+
+mvd_status build_compounds(int n_views, const float* d_psf, const long* koff, const int* kd, int variant, float* d_out,
+                           const float* d_q, long qstride, float* d_c, int group, int* d_bad, cudaStream_t st) {
+    const bool pairs = (variant == MVD_EFFICIENT || variant == MVD_OPT1) && n_views > 1;
+    for (int first = 0; first < n_views; first += group) {
+        const int last = first + group < n_views ? first + group : n_views;
+        std::vector<BoxJob> jobs;
+        std::vector<float*> cv(last - first, nullptr);
+        float* c = d_c;
+        for (int v = first; v < last && pairs; ++v) {
+            const int* k = kd + 3 * v;
+            const size_t T = (size_t)k[0] * k[1] * k[2];
+            cv[v - first] = c;
+            for (int w = 0; w < n_views; ++w) {
+                if (w == v) continue;
+                // C_w(d) = sum_e P_v^*(e) G(d - e) = sum_t P_v(t) G(d + t), G = Q_w or P_w
+                const int* kw = kd + 3 * w;
+                const bool eff = variant == MVD_EFFICIENT;
+                const int gd[3] = {eff ? 2 * kw[0] - 1 : kw[0], eff ? 2 * kw[1] - 1 : kw[1], eff ? 2 * kw[2] - 1 : kw[2]};
+                const float* G = eff ? d_q + (size_t)w * qstride : d_psf + koff[w];
+                jobs.push_back(box_job(G, gd, d_psf + koff[v], k, false, c, k));
+                c += T;
             }
+        }
+        MVD_TRY(box_convs(std::move(jobs), st));
+        for (int v0 = first; v0 < last; v0 += kFinishViews) {
+            FinishArgs a{};
+            const int n = last - v0 < kFinishViews ? last - v0 : kFinishViews;
+            for (int i = 0; i < n; ++i)
+                a.v[i] = Finish{d_psf + koff[v0 + i], cv[v0 + i - first], d_out + koff[v0 + i], box_of(kd + 3 * (v0 + i))};
+            k_compound_finish<<<n, 1024, 0, st>>>(a, variant == MVD_PLAIN ? 0 : n_views - 1, d_bad);
             count_launch();
             MVD_TRY(check_launch("compound product"));
         }
@@ -272,20 +284,6 @@ mvd_status mirror_kernel(const float* k, const int kd[3], float* out, cudaStream
     k_mirror<<<blocks_for((long)b.kx * b.ky * b.kz), kThreads, 0, st>>>(k, b, out);
     count_launch();
     return check_launch("mirror kernel");
-}
-
-mvd_status autocorr_kernel(const float* P, const int kd[3], float* Q, cudaStream_t st) {
-    const Box b = box_of(kd);
-    const Box q{2 * b.kx - 1, 2 * b.ky - 1, 2 * b.kz - 1};
-    k_autocorr<<<warp_blocks_for((long)q.kx * q.ky * q.kz), kThreads, 0, st>>>(P, b, Q, q);
-    count_launch();
-    return check_launch("autocorrelation");
-}
-
-mvd_status normalize_kernel(float* d_k, int n, int* d_bad, cudaStream_t st) {
-    k_normalize<<<1, 1024, 0, st>>>(d_k, n, d_bad);
-    count_launch();
-    return check_launch("normalise kernel");
 }
 
 mvd_status place_kernel(const int dims[3], const float* k, const int kd[3], float* vol, cudaStream_t st) {
