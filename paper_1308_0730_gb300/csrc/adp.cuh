@@ -1,0 +1,256 @@
+// Aligned double-float (adf.cuh) on packed pairs: a complex value is two 64-bit
+// register pairs, the high parts (re, im) and the low parts (re, im), and every
+// operation is one two-lane FP32 instruction (add/mul/fma.rn.f32x2, each lane
+// rounded as its scalar form). The steps are those of adf.cuh, operation for
+// operation, so the results are bit-identical to it.
+//
+// Why: the FFT passes are bound by issue slots and shared memory, not by the FP32
+// lanes. One radix-8 stage with its twiddles takes 23 instructions per point
+// against 42 in scalar form; alone it runs at 117 lanes per clock and SM (the
+// FP32 peak) and 2.93 points per clock against 2.42. The exchange of re and im that a
+// product by i needs and the broadcast of a twiddle's part to both lanes cost almost
+// nothing (operand selection). Packing two lines instead of re and im gave the same
+// rate for twice the registers.
+//
+// In memory (global and shared) a complex double-float is 16 bytes in the order
+// re.hi, im.hi, re.lo, im.lo, so that a 16-byte load gives the two pairs.
+#pragma once
+
+#include "dd.cuh"
+
+namespace mvd {
+
+typedef unsigned long long f2;  // two FP32 lanes: low word = first
+
+__device__ __forceinline__ f2 f2_of(float a, float b) {
+    f2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void f2_get(f2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 f2_neg(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2 f2_swap(f2 a) {
+    float x, y;
+    f2_get(a, x, y);
+    return f2_of(y, x);
+}
+__device__ __forceinline__ f2 f2_dup(float a) { return f2_of(a, a); }
+
+// complex double-float: h = (re.hi, im.hi), l = (re.lo, im.lo)
+struct cdp {
+    f2 h, l;
+};
+
+__device__ __forceinline__ cdp cdp_from4(float4 v) { return {f2_of(v.x, v.y), f2_of(v.z, v.w)}; }
+__device__ __forceinline__ cdp cdp_load(const cdd* p) { return cdp_from4(*reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ cdp cdp_load_cg(const cdd* p) { return cdp_from4(__ldcg(reinterpret_cast<const float4*>(p))); }
+__device__ __forceinline__ cdp cdp_load_nc(const cdd* p) { return cdp_from4(__ldg(reinterpret_cast<const float4*>(p))); }
+__device__ __forceinline__ void cdp_store(cdd* p, cdp a) {
+    float4 v;
+    f2_get(a.h, v.x, v.y);
+    f2_get(a.l, v.z, v.w);
+    *reinterpret_cast<float4*>(p) = v;
+}
+__device__ __forceinline__ cdp cdp_zero() { return {0ull, 0ull}; }
+__device__ __forceinline__ cdp cdp_from(float re, float im) { return {f2_of(re, im), 0ull}; }
+// the value rounded to FP32 (re, im)
+__device__ __forceinline__ float2 cdp_round(cdp a) {
+    float x, y;
+    f2_get(f2_add(a.h, a.l), x, y);
+    return make_float2(x, y);
+}
+__device__ __forceinline__ float cdp_absmax(cdp a, float m) {
+    float x, y;
+    f2_get(a.h, x, y);
+    return fmaxf(m, fmaxf(fabsf(x), fabsf(y)));
+}
+
+__device__ __forceinline__ cdp cdp_add(cdp a, cdp b) { return {f2_add(a.h, b.h), f2_add(a.l, b.l)}; }
+__device__ __forceinline__ cdp cdp_sub(cdp a, cdp b) { return {f2_sub(a.h, b.h), f2_sub(a.l, b.l)}; }
+__device__ __forceinline__ cdp cdp_half(cdp a) {  // exact
+    const f2 k = f2_dup(0.5f);
+    return {f2_mul(a.h, k), f2_mul(a.l, k)};
+}
+// the sign pair of a product by s i: s i (x + i y) = (-s y) + i (s x)
+template <int S>
+__device__ __forceinline__ f2 f2_si() {
+    return f2_of(S > 0 ? -1.f : 1.f, S > 0 ? 1.f : -1.f);
+}
+// a + S i b (exact product by +-1, then the same rounding as an add)
+template <int S>
+__device__ __forceinline__ cdp cdp_addi(cdp a, cdp b) {
+    const f2 s = f2_si<S>();
+    return {f2_fma(f2_swap(b.h), s, a.h), f2_fma(f2_swap(b.l), s, a.l)};
+}
+template <int S>
+__device__ __forceinline__ cdp cdp_muli(cdp a) {  // S i a, exact
+    const f2 s = f2_si<S>();
+    return {f2_mul(f2_swap(a.h), s), f2_mul(f2_swap(a.l), s)};
+}
+__device__ __forceinline__ cdp cdp_neg(cdp a) { return {f2_neg(a.h), f2_neg(a.l)}; }
+__device__ __forceinline__ cdp cdp_conj(cdp a) {
+    return {a.h ^ 0x8000000000000000ull, a.l ^ 0x8000000000000000ull};
+}
+
+// onto the grid of the constant pair c (adf_align)
+__device__ __forceinline__ cdp cdp_align(cdp x, f2 c) {
+    const f2 h = f2_sub(f2_add(x.h, c), c);
+    return {h, f2_add(f2_sub(x.h, h), x.l)};
+}
+// lane-wise products by the double-float constants (kh + kl), aligned (adf_mulk)
+__device__ __forceinline__ cdp cdp_mulk(cdp a, f2 kh, f2 kl, f2 c) {
+    const f2 h = f2_sub(f2_add(f2_mul(a.h, kh), c), c);
+    f2 r = f2_fma(a.h, kh, f2_neg(h));
+    r = f2_fma(a.h, kl, r);
+    return {h, f2_fma(a.l, kh, r)};
+}
+__device__ __forceinline__ cdp cdp_mulk(cdp a, dd k, f2 c) { return cdp_mulk(a, f2_dup(k.hi), f2_dup(k.lo), c); }
+// by an FP32-exact constant (adf_mulf)
+__device__ __forceinline__ cdp cdp_mulf(cdp a, float k, f2 c) {
+    const f2 kk = f2_dup(k), h = f2_sub(f2_add(f2_mul(a.h, kk), c), c);
+    return {h, f2_fma(a.l, kk, f2_fma(a.h, kk, f2_neg(h)))};
+}
+// x w (S < 0) or x conj(w) (S > 0), w a forward twiddle, aligned (adf_cmul): 14 instructions
+template <int S>
+__device__ __forceinline__ cdp cdp_cmul(cdp x, cdp w, f2 c) {
+    float rh, ih, rl, il;
+    f2_get(w.h, rh, ih);
+    f2_get(w.l, rl, il);
+    const cdp xs{f2_swap(x.h), f2_swap(x.l)};
+    const cdp q = S < 0 ? cdp_mulk(xs, f2_of(-ih, ih), f2_of(-il, il), c) : cdp_mulk(xs, f2_of(ih, -ih), f2_of(il, -il), c);
+    return cdp_add(cdp_mulk(x, f2_dup(rh), f2_dup(rl), c), q);
+}
+
+// double-float sums without a grid (dd_add: TwoSum of the high parts, 8 instructions)
+__device__ __forceinline__ cdp cdp_two_add(cdp x, cdp y) {
+    const f2 s = f2_add(x.h, y.h), bb = f2_sub(s, x.h);
+    const f2 e = f2_add(f2_sub(x.h, f2_sub(s, bb)), f2_sub(y.h, bb));
+    return {s, f2_add(e, f2_add(x.l, y.l))};
+}
+// x y as an unevaluated pair (dd_dot2_pair): 16 instructions
+__device__ __forceinline__ cdp cdp_mul_pair(cdp x, cdp y) {
+    float rh, ih, rl, il;
+    f2_get(y.h, rh, ih);
+    f2_get(y.l, rl, il);
+    const f2 xs = f2_swap(x.h), rr = f2_dup(rh), ii = f2_of(-ih, ih);
+    const f2 p = f2_mul(x.h, rr), q = f2_mul(xs, ii);
+    f2 e = f2_fma(x.h, rr, f2_neg(p)), f = f2_fma(xs, ii, f2_neg(q));
+    e = f2_fma(x.h, f2_dup(rl), e);
+    e = f2_fma(x.l, rr, e);
+    f = f2_fma(xs, f2_of(-il, il), f);
+    f = f2_fma(f2_swap(x.l), ii, f);
+    const f2 s = f2_add(p, q), bb = f2_sub(s, p);
+    const f2 t = f2_add(f2_sub(p, f2_sub(s, bb)), f2_sub(q, bb));
+    return {s, f2_add(t, f2_add(e, f))};
+}
+
+// x s for a real double-float s, renormalised (dd_mul)
+__device__ __forceinline__ cdp cdp_scale(cdp x, dd s) {
+    const f2 sh = f2_dup(s.hi), p = f2_mul(x.h, sh);
+    f2 e = f2_fma(x.h, sh, f2_neg(p));
+    e = f2_fma(x.h, f2_dup(s.lo), e);
+    e = f2_fma(x.l, sh, e);
+    const f2 h = f2_add(p, e);
+    return {h, f2_sub(e, f2_sub(h, p))};
+}
+
+// small DFTs on aligned values (DftA of adf.cuh)
+template <int R, int S>
+struct DftP;
+
+template <int S>
+struct DftP<2, S> {
+    __device__ __forceinline__ static void run(cdp* v, f2) {
+        const cdp a = v[0], b = v[1];
+        v[0] = cdp_add(a, b);
+        v[1] = cdp_sub(a, b);
+    }
+};
+
+template <int S>
+struct DftP<4, S> {
+    __device__ __forceinline__ static void run(cdp* v, f2) {
+        const cdp t0 = cdp_add(v[0], v[2]), t1 = cdp_sub(v[0], v[2]);
+        const cdp t2 = cdp_add(v[1], v[3]), t3 = cdp_sub(v[1], v[3]);
+        v[0] = cdp_add(t0, t2);
+        v[2] = cdp_sub(t0, t2);
+        v[1] = cdp_addi<S>(t1, t3);
+        v[3] = cdp_addi<-S>(t1, t3);
+    }
+};
+
+template <int S>
+struct DftP<8, S> {
+    __device__ __forceinline__ static void run(cdp* v, f2 c) {
+        cdp e[4] = {v[0], v[2], v[4], v[6]};
+        cdp o[4] = {v[1], v[3], v[5], v[7]};
+        DftP<4, S>::run(e, c);
+        DftP<4, S>::run(o, c);
+        // o1 (1 + S i) h and o3 (-1 + S i) h, h = sqrt(2)/2
+        const dd hd = MVD_DD(0.70710678118654752440);
+        const cdp w1 = cdp_mulk(cdp_addi<S>(o[1], o[1]), hd, c);
+        const cdp w3 = cdp_mulk(cdp_addi<-S>(o[3], o[3]), hd, c);  // its negative
+        v[0] = cdp_add(e[0], o[0]);
+        v[4] = cdp_sub(e[0], o[0]);
+        v[1] = cdp_add(e[1], w1);
+        v[5] = cdp_sub(e[1], w1);
+        v[2] = cdp_addi<S>(e[2], o[2]);
+        v[6] = cdp_addi<-S>(e[2], o[2]);
+        v[3] = cdp_sub(e[3], w3);
+        v[7] = cdp_add(e[3], w3);
+    }
+};
+
+template <int S>
+struct DftP<3, S> {
+    __device__ __forceinline__ static void run(cdp* v, f2 c) {
+        const cdp t = cdp_add(v[1], v[2]), u = cdp_sub(v[1], v[2]);
+        const dd hd = MVD_DD(0.86602540378443864676);  // sin(2 pi / 3)
+        const cdp m = cdp_add(v[0], cdp_mulf(t, -0.5f, c)), j = cdp_mulk(u, hd, c);
+        v[0] = cdp_add(v[0], t);
+        v[1] = cdp_addi<S>(m, j);
+        v[2] = cdp_addi<-S>(m, j);
+    }
+};
+
+template <int S>
+struct DftP<5, S> {
+    __device__ __forceinline__ static void run(cdp* v, f2 c) {
+        const dd c1 = MVD_DD(0.30901699437494742410), c2 = MVD_DD(-0.80901699437494742410);
+        const dd s1 = MVD_DD(0.95105651629515357212), s2 = MVD_DD(0.58778525229247312917);
+        const cdp t1 = cdp_add(v[1], v[4]), u1 = cdp_sub(v[1], v[4]);
+        const cdp t2 = cdp_add(v[2], v[3]), u2 = cdp_sub(v[2], v[3]);
+        const cdp a0 = v[0];
+        const cdp m1 = cdp_add(a0, cdp_add(cdp_mulk(t1, c1, c), cdp_mulk(t2, c2, c)));
+        const cdp m2 = cdp_add(a0, cdp_add(cdp_mulk(t1, c2, c), cdp_mulk(t2, c1, c)));
+        const cdp j1 = cdp_add(cdp_mulk(u1, s1, c), cdp_mulk(u2, s2, c));
+        const cdp j2 = cdp_sub(cdp_mulk(u1, s2, c), cdp_mulk(u2, s1, c));
+        v[0] = cdp_add(a0, cdp_add(t1, t2));
+        v[1] = cdp_addi<S>(m1, j1);
+        v[4] = cdp_addi<-S>(m1, j1);
+        v[2] = cdp_addi<S>(m2, j2);
+        v[3] = cdp_addi<-S>(m2, j2);
+    }
+};
+
+}  // namespace mvd

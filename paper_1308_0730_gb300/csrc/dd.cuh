@@ -48,7 +48,9 @@ __device__ __forceinline__ dd dd_mul(dd x, dd y) {
 }
 __device__ __forceinline__ dd dd_from(float a) { return {a, 0.f}; }
 
-// complex double-float, 16 bytes (loads and stores as float4)
+// complex double-float, 16 bytes. In device memory (global and shared) the order is
+// re.hi, im.hi, re.lo, im.lo (adp.cuh): use cdd_load / cdd_store, never a plain copy
+// of the struct.
 struct __align__(16) cdd {
     dd re, im;
 };
@@ -102,18 +104,18 @@ __device__ __forceinline__ cdd mul_si(cdd a) {  // exact
 __device__ __forceinline__ cdd czero_dd() { return {dd{0.f, 0.f}, dd{0.f, 0.f}}; }
 __device__ __forceinline__ cdd cdd_load(const cdd* p) {
     const float4 v = *reinterpret_cast<const float4*>(p);
-    return {dd{v.x, v.y}, dd{v.z, v.w}};
+    return {dd{v.x, v.z}, dd{v.y, v.w}};
 }
 __device__ __forceinline__ cdd cdd_load_cg(const cdd* p) {
     const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
-    return {dd{v.x, v.y}, dd{v.z, v.w}};
+    return {dd{v.x, v.z}, dd{v.y, v.w}};
 }
 __device__ __forceinline__ cdd cdd_load_nc(const cdd* p) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-    return {dd{v.x, v.y}, dd{v.z, v.w}};
+    return {dd{v.x, v.z}, dd{v.y, v.w}};
 }
 __device__ __forceinline__ void cdd_store(cdd* p, cdd a) {
-    *reinterpret_cast<float4*>(p) = make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo);
+    *reinterpret_cast<float4*>(p) = make_float4(a.re.hi, a.im.hi, a.re.lo, a.im.lo);
 }
 
 // 16-byte asynchronous global -> shared copy (L2 only); with !valid nothing is

@@ -58,11 +58,11 @@ __device__ __forceinline__ void stockham_stage_dd(const cdd* __restrict__ A, cdd
         cdd* b = B + line * ls;
         cdd v[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = a[j + r * si.nb];
+        for (int r = 0; r < R; ++r) v[r] = cdd_load(a + j + r * si.nb);
         dd_bfly_math<R, S, ALN>(v, k, si, tw, c, mx);
         const int d = jq * si.Ns * R + k;
 #pragma unroll
-        for (int r = 0; r < R; ++r) b[d + r * si.Ns] = v[r];
+        for (int r = 0; r < R; ++r) cdd_store(b + d + r * si.Ns, v[r]);
     }
 }
 
@@ -98,7 +98,7 @@ __device__ __forceinline__ void stockham_stage_dd_io(const cdd* __restrict__ A, 
                 const cdd* q = gin + (long)line * gls + (long)(j + r * si.nb) * ges;
                 v[r] = ok ? (CO ? cdd_load_cg(q) : cdd_load(q)) : czero_dd();
             } else {
-                v[r] = A[line * ls + j + r * si.nb];
+                v[r] = cdd_load(A + line * ls + j + r * si.nb);
             }
         }
         dd_bfly_math<R, S, ALN>(v, k, si, tw, c, mx);
@@ -108,7 +108,7 @@ __device__ __forceinline__ void stockham_stage_dd_io(const cdd* __restrict__ A, 
             if (GOUT) {
                 if (ok) cdd_store(gout + (long)line * gls + (long)(d + r * si.Ns) * ges, v[r]);
             } else {
-                B[line * ls + d + r * si.Ns] = v[r];
+                cdd_store(B + line * ls + d + r * si.Ns, v[r]);
             }
         }
     }
@@ -293,7 +293,7 @@ __device__ void dd_x_forward_tile(const DdX& a, long tile, cdd* sm) {
         const int p = t / a.X, n = t - p * a.X;
         const float va = p < nrows ? ld1<CO>(a.src + (rho0 + p) * a.X + n) : 0.f;
         const float vb = a.P + p < nrows ? ld1<CO>(a.src + (rho0 + a.P + p) * a.X + n) : 0.f;
-        A[p * a.ls + n] = cdd{dd_from(va), dd_from(vb)};
+        cdd_store(A + p * a.ls + n, cdd{dd_from(va), dd_from(vb)});
     }
     __syncthreads();
     const cdd* F = fft_lines_dd<-1>(A, B, a.P, a.ls, a.plan, a.tw2);
@@ -302,8 +302,8 @@ __device__ void dd_x_forward_tile(const DdX& a, long tile, cdd* sm) {
         const int k = t / P2, row = t - k * P2;
         if (row >= nrows) continue;
         const int p = row < a.P ? row : row - a.P;
-        const cdd zk = F[p * a.ls + k];
-        const cdd zm = cconj(F[p * a.ls + (k == 0 ? 0 : a.X - k)]);
+        const cdd zk = cdd_load(F + p * a.ls + k);
+        const cdd zm = cconj(cdd_load(F + p * a.ls + (k == 0 ? 0 : a.X - k)));
         cdd val;
         if (row < a.P) {
             val = chalf(cadd(zk, zm));
@@ -327,8 +327,8 @@ __device__ __forceinline__ void dd_x_unpack_store(const DdX& a, const cdd* F, lo
         const int k = t / P2, row = t - k * P2;
         if (row >= nrows) continue;
         const int p = row < a.P ? row : row - a.P;
-        const cdd zk = F[p * a.ls + k];
-        const cdd zm = cconj(F[p * a.ls + (k == 0 ? 0 : a.X - k)]);
+        const cdd zk = cdd_load(F + p * a.ls + k);
+        const cdd zm = cconj(cdd_load(F + p * a.ls + (k == 0 ? 0 : a.X - k)));
         cdd val;
         if (row < a.P) {
             val = chalf(cadd(zk, zm));
@@ -350,17 +350,17 @@ __device__ __forceinline__ void dd_x_gather_lines(const DdX& a, cdd* A, cdd* B, 
         cdd v = czero_dd();
         if (row < nrows) v = CO ? cdd_load_cg(a.S2 + (long)k * a.YZ + rho0 + row) : cdd_load(a.S2 + (long)k * a.YZ + rho0 + row);
         if (row < a.P)
-            A[row * a.ls + k] = v;
+            cdd_store(A + row * a.ls + k, v);
         else
-            B[(row - a.P) * a.ls + k] = v;
+            cdd_store(B + (row - a.P) * a.ls + k, v);
     }
     __syncthreads();
     const int half = (a.X + 1) / 2;
     for (int t = threadIdx.x; t < a.P * a.Xh; t += blockDim.x) {
         const int p = t / a.Xh, k = t - p * a.Xh;
-        const cdd av = A[p * a.ls + k], bv = B[p * a.ls + k];
-        A[p * a.ls + k] = cdd{dd_sub(av.re, bv.im), dd_add(av.im, bv.re)};
-        if (k >= 1 && k < half) A[p * a.ls + (a.X - k)] = cdd{dd_add(av.re, bv.im), dd_sub(bv.re, av.im)};
+        const cdd av = cdd_load(A + p * a.ls + k), bv = cdd_load(B + p * a.ls + k);
+        cdd_store(A + p * a.ls + k, cdd{dd_sub(av.re, bv.im), dd_add(av.im, bv.re)});
+        if (k >= 1 && k < half) cdd_store(A + p * a.ls + (a.X - k), cdd{dd_add(av.re, bv.im), dd_sub(bv.re, av.im)});
     }
     __syncthreads();
 }
@@ -389,7 +389,7 @@ __device__ void dd_x_update_tile(const DdXU& u, long tile, cdd* sm) {
     const int n2 = a.P * a.X;
     for (int t = threadIdx.x; t < n2; t += blockDim.x) {
         const int p = t / a.X, n = t - p * a.X;
-        const cdd z = R[p * a.ls + n];
+        const cdd z = cdd_load(R + p * a.ls + n);
         const float cv[2] = {z.re.hi + z.re.lo, z.im.hi + z.im.lo};  // c - 1 of rows p and P + p
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -421,18 +421,18 @@ __device__ void dd_x_ratio_tile(const DdX& a, long tile, cdd* sm) {
         cdd v = czero_dd();
         if (row < nrows) v = CO ? cdd_load_cg(a.S2 + (long)k * a.YZ + rho0 + row) : cdd_load(a.S2 + (long)k * a.YZ + rho0 + row);
         if (row < a.P)
-            A[row * a.ls + k] = v;
+            cdd_store(A + row * a.ls + k, v);
         else
-            B[(row - a.P) * a.ls + k] = v;
+            cdd_store(B + (row - a.P) * a.ls + k, v);
     }
     __syncthreads();
     const int half = (a.X + 1) / 2;
     for (int t = threadIdx.x; t < a.P * a.Xh; t += blockDim.x) {
         const int p = t / a.Xh, k = t - p * a.Xh;
-        const cdd av = A[p * a.ls + k], bv = B[p * a.ls + k];
+        const cdd av = cdd_load(A + p * a.ls + k), bv = cdd_load(B + p * a.ls + k);
         // A + iB and, at -k, conj(A) + i conj(B)
-        A[p * a.ls + k] = cdd{dd_sub(av.re, bv.im), dd_add(av.im, bv.re)};
-        if (k >= 1 && k < half) A[p * a.ls + (a.X - k)] = cdd{dd_add(av.re, bv.im), dd_sub(bv.re, av.im)};
+        cdd_store(A + p * a.ls + k, cdd{dd_sub(av.re, bv.im), dd_add(av.im, bv.re)});
+        if (k >= 1 && k < half) cdd_store(A + p * a.ls + (a.X - k), cdd{dd_add(av.re, bv.im), dd_sub(bv.re, av.im)});
     }
     __syncthreads();
     cdd* R = fft_lines_dd<+1>(A, B, a.P, a.ls, a.plan, a.tw2);
@@ -442,7 +442,7 @@ __device__ void dd_x_ratio_tile(const DdX& a, long tile, cdd* sm) {
     const int n2 = a.P * a.X;
     for (int t = threadIdx.x; t < n2; t += blockDim.x) {
         const int p = t / a.X, n = t - p * a.X;
-        const cdd z = R[p * a.ls + n];
+        const cdd z = cdd_load(R + p * a.ls + n);
         const float ba = z.re.hi + z.re.lo, bb = z.im.hi + z.im.lo;
         float ra = 0.f, rb = 0.f;
         if (p < nrows) ra = __ldg(a.phi + (rho0 + p) * a.X + n) / fmaxf(ba, a.eps) - 1.f;
@@ -516,13 +516,13 @@ __device__ void dd_y_tile(const DdY& a, long tile, cdd* sm) {
         const int line = t / a.L, y = t - line * a.L;
         cdd v = czero_dd();
         if (line < nl) v = CO ? cdd_load_cg(a.S2 + (l0 + line) * a.L + y) : cdd_load(a.S2 + (l0 + line) * a.L + y);
-        A[line * a.ls + y] = v;
+        cdd_store(A + line * a.ls + y, v);
     }
     __syncthreads();
     const cdd* R = fft_lines_dd<S>(A, B, a.P, a.ls, a.plan, a.tw2);
     for (int t = threadIdx.x; t < nl * a.L; t += blockDim.x) {
         const int line = t / a.L, y = t - line * a.L;
-        cdd_store(a.S2 + (l0 + line) * a.L + y, R[line * a.ls + y]);
+        cdd_store(a.S2 + (l0 + line) * a.L + y, cdd_load(R + line * a.ls + y));
     }
 }
 
@@ -575,7 +575,7 @@ __device__ void dd_z_tile(const DdZ& a, long tile, cdd* sm) {
         cdd* F = fft_lines_dd_io<-1, false, false, CO, true>(a.S2 + base, 1, a.Y, A, B, a.Q, nq, a.ls, a.plan, a.tw2);
         for (int t = threadIdx.x; t < n; t += blockDim.x) {
             const int z = t / a.Q, q = t - z * a.Q;
-            if (q < nq) F[q * a.ls + z] = cmul(F[q * a.ls + z], cdd_load_nc(a.K2 + base + (long)z * a.Y + q));
+            if (q < nq) cdd_store(F + q * a.ls + z, cmul(cdd_load(F + q * a.ls + z), cdd_load_nc(a.K2 + base + (long)z * a.Y + q)));
         }
         __syncthreads();
         fft_lines_dd_io<+1, false, true, CO, true>(a.S2 + base, 1, a.Y, F, F == A ? B : A, a.Q, nq, a.ls, a.plan,
@@ -586,7 +586,7 @@ __device__ void dd_z_tile(const DdZ& a, long tile, cdd* sm) {
         const int z = t / a.Q, q = t - z * a.Q;
         cdd v = czero_dd();
         if (q < nq) v = CO ? cdd_load_cg(a.S2 + base + (long)z * a.Y + q) : cdd_load(a.S2 + base + (long)z * a.Y + q);
-        A[q * a.ls + z] = v;
+        cdd_store(A + q * a.ls + z, v);
     }
     __syncthreads();
     cdd* F = fft_lines_dd<-1>(A, B, a.Q, a.ls, a.plan, a.tw2);
@@ -594,7 +594,7 @@ __device__ void dd_z_tile(const DdZ& a, long tile, cdd* sm) {
     if (MUL) {
         for (int t = threadIdx.x; t < n; t += blockDim.x) {
             const int z = t / a.Q, q = t - z * a.Q;
-            if (q < nq) F[q * a.ls + z] = cmul(F[q * a.ls + z], cdd_load_nc(a.K2 + base + (long)z * a.Y + q));
+            if (q < nq) cdd_store(F + q * a.ls + z, cmul(cdd_load(F + q * a.ls + z), cdd_load_nc(a.K2 + base + (long)z * a.Y + q)));
         }
         __syncthreads();
         F = fft_lines_dd<+1>(F, O, a.Q, a.ls, a.plan, a.tw2);
@@ -602,7 +602,7 @@ __device__ void dd_z_tile(const DdZ& a, long tile, cdd* sm) {
     for (int t = threadIdx.x; t < n; t += blockDim.x) {
         const int z = t / a.Q, q = t - z * a.Q;
         if (q < nq) {
-            cdd v = F[q * a.ls + z];
+            cdd v = cdd_load(F + q * a.ls + z);
             if (!MUL) v = cdd{dd_mul(v.re, a.scale), dd_mul(v.im, a.scale)};
             cdd_store(a.S2 + base + (long)z * a.Y + q, v);
         }

@@ -6,6 +6,7 @@
 #pragma once
 
 #include "adf.cuh"
+#include "adp.cuh"
 #include "dd.cuh"
 #include "fft_fast.cuh"
 
@@ -51,7 +52,7 @@ __host__ __device__ constexpr int tw_stage_off(int L, int ST) {
 __device__ __forceinline__ int pad8(int i) { return i + (i >> 3); }
 __host__ __device__ constexpr int line_stride8(int L) { return L + L / 8 + 1; }
 
-// Arithmetic: aligned double-float (adf.cuh). run() first takes the largest
+// Arithmetic: aligned double-float on packed pairs (adf.cuh, adp.cuh). run() first takes the largest
 // component of the line (a reduction over its threads), puts every value on
 // the grid of that bound's quantum, and each later stage moves to a grid 16
 // times coarser (the growth bound of a radix-8 stage); butterfly sums are then
@@ -92,10 +93,10 @@ struct LineFFTDD {
     }
 
     // largest |hi| component over the line's TPL threads
-    __device__ __forceinline__ static float line_bound(const cdd (&v)[kE8], cdd* sm, int t, int bar) {
+    __device__ __forceinline__ static float line_bound(const cdp (&v)[kE8], cdd* sm, int t, int bar) {
         float m = 0.f;
 #pragma unroll
-        for (int q = 0; q < kE8; ++q) m = adf_absmax(v[q], m);
+        for (int q = 0; q < kE8; ++q) m = cdp_absmax(v[q], m);
         if constexpr (WARP_LOCAL) {
             constexpr int W = TPL < 32 ? TPL : 32;
 #pragma unroll
@@ -121,36 +122,34 @@ struct LineFFTDD {
     }
 
     template <int ST, int NS>
-    __device__ __forceinline__ static void stage(cdd (&v)[kE8], cdd* sm, int t, const cdd* __restrict__ tw, int bar,
+    __device__ __forceinline__ static void stage(cdp (&v)[kE8], cdd* sm, int t, const cdd* __restrict__ tw, int bar,
                                                  int e0) {
         if constexpr (ST < NST) {
             constexpr int R = plan8_radix(L, ST);
             constexpr int B = kE8 / R;
             constexpr bool LAST = (ST == NST - 1);
-            const float c = adf_const_exp2(e0 + 4 * ST);  // every stage before this one is radix 8
+            const f2 c = f2_dup(adf_const_exp2(e0 + 4 * ST));  // every stage before this one is radix 8
 #pragma unroll
             for (int m = 0; m < B; ++m) {
-                cdd x[R];
+                cdp x[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) x[r] = v[m + r * B];
                 const int j = t + TPL * m;
                 const int k = j % NS;
                 if (NS > 1) {
                     constexpr int OFF = tw_stage_off(L, ST);
-                    x[0] = adf_calign(x[0], c);
+                    x[0] = cdp_align(x[0], c);
 #pragma unroll
                     for (int r = 1; r < R; ++r) {
-                        cdd w;
-                        if constexpr (TWS) {
-                            w = cdd_load(tw + pad8(OFF + (r - 1) * NS + k));
-                            if (S > 0) w.im = dd{-w.im.hi, -w.im.lo};
-                        } else {
-                            w = twiddle_dd<S>(tw + L, OFF + (r - 1) * NS + k);
-                        }
-                        x[r] = adf_cmul(x[r], w, c);
+                        cdp w;
+                        if constexpr (TWS)
+                            w = cdp_load(tw + pad8(OFF + (r - 1) * NS + k));
+                        else
+                            w = cdp_load_nc(tw + L + OFF + (r - 1) * NS + k);
+                        x[r] = cdp_cmul<S>(x[r], w, c);
                     }
                 }
-                DftA<R, S>::run(x, c);
+                DftP<R, S>::run(x, c);
                 if (LAST) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) v[m + r * B] = x[r];
@@ -158,14 +157,14 @@ struct LineFFTDD {
                     const int d = (j / NS) * NS * R + k;
                     cdd* buf = sm + ((DB > 0 && (ST & 1)) ? DB : 0);
 #pragma unroll
-                    for (int r = 0; r < R; ++r) cdd_store(buf + pad8(d + r * NS), x[r]);
+                    for (int r = 0; r < R; ++r) cdp_store(buf + pad8(d + r * NS), x[r]);
                 }
             }
             if constexpr (!LAST) {
                 const cdd* buf = sm + ((DB > 0 && (ST & 1)) ? DB : 0);
                 sync(bar);
 #pragma unroll
-                for (int q = 0; q < kE8; ++q) v[q] = cdd_load(buf + pad8(t + TPL * q));
+                for (int q = 0; q < kE8; ++q) v[q] = cdp_load(buf + pad8(t + TPL * q));
                 if constexpr (DB == 0) sync(bar);
                 stage<ST + 1, NS * R>(v, sm, t, tw, bar, e0);
             }
@@ -173,15 +172,20 @@ struct LineFFTDD {
     }
 
     // bar: the line's named barrier (1 + its index in the block) when WARP_LOCAL
-    __device__ __forceinline__ static void run(cdd (&v)[kE8], cdd* sm, int t, const cdd* __restrict__ tw,
+    __device__ __forceinline__ static void run(cdp (&v)[kE8], cdd* sm, int t, const cdd* __restrict__ tw,
                                                int bar = 1) {
         const int e0 = adf_exp_for(line_bound(v, sm, t, bar));
-        const float c0 = adf_const_exp2(e0);
+        const f2 c0 = f2_dup(adf_const_exp2(e0));
 #pragma unroll
-        for (int q = 0; q < kE8; ++q) v[q] = adf_calign(v[q], c0);
+        for (int q = 0; q < kE8; ++q) v[q] = cdp_align(v[q], c0);
         stage<0, 1>(v, sm, t, tw, bar, e0);
     }
 };
+
+// Measured with the packed pairs against scalar aligned double-float (per launch, us):
+// 256x256x128: a view update 302 -> 277; 1024x1024x512: y 1674 -> 1589, z 3490 -> 3357. Issue slots busy 57-72% ->
+// 38-59%; the L1 pipe (exchanges and twiddles, 65-93% busy in the x and y passes) and,
+// in z, the warps in flight bound them now.
 
 // The same register-resident plan in FP32 (float2 elements; tw is the FP32
 // natural table of L, followed by its radix-8 stage-ordered copy): used for
@@ -287,11 +291,11 @@ __host__ __device__ constexpr size_t ddf_z_smem(int L) {
 }
 
 template <bool CO>
-__device__ __forceinline__ cdd ld_cdd(const cdd* p) {
+__device__ __forceinline__ cdp ld_cdp(const cdd* p) {
     if constexpr (CO)
-        return cdd_load_cg(p);
+        return cdp_load_cg(p);
     else
-        return cdd_load(p);
+        return cdp_load(p);
 }
 
 // IO selects where the lines come from:
@@ -309,20 +313,20 @@ __device__ __forceinline__ void ddf_y_tile(cdd* __restrict__ S2, long nlines, co
     const bool ok = line < nlines;
     cdd* g = S2 + line * L;
     float2* g1 = S1 + line * L;
-    cdd v[kE8];
+    cdp v[kE8];
 #pragma unroll
     for (int q = 0; q < kE8; ++q) {
         if constexpr (IO == 1) {
             const float2 f = ok ? (CO ? __ldcg(g1 + t + TPL * q) : g1[t + TPL * q]) : make_float2(0.f, 0.f);
-            v[q] = cdd{dd_from(f.x), dd_from(f.y)};
+            v[q] = cdp_from(f.x, f.y);
         } else {
-            v[q] = ok ? ld_cdd<CO>(g + t + TPL * q) : czero_dd();
+            v[q] = ok ? ld_cdp<CO>(g + t + TPL * q) : cdp_zero();
         }
     }
     F::run(v, sm + li * line_stride8(L), t, tw2, 1 + li);
     if (ok) {
 #pragma unroll
-        for (int q = 0; q < kE8; ++q) cdd_store(g + t + TPL * q, v[q]);
+        for (int q = 0; q < kE8; ++q) cdp_store(g + t + TPL * q, v[q]);
     }
 }
 
@@ -338,24 +342,24 @@ __device__ __forceinline__ void ddf_z_tile(cdd* __restrict__ S2, const cdd* __re
     const bool ok = y0 + q < Y;
     const long base = (long)kx * YZ + y0 + q;
     cdd* line_sm = sm + q * z_line_stride8(L);
-    cdd v[kE8];
+    cdp v[kE8];
 #pragma unroll
-    for (int i = 0; i < kE8; ++i) v[i] = ok ? ld_cdd<CO>(S2 + base + (long)(t + TPL * i) * Y) : czero_dd();
+    for (int i = 0; i < kE8; ++i) v[i] = ok ? ld_cdp<CO>(S2 + base + (long)(t + TPL * i) * Y) : cdp_zero();
     using FF = LineFFTDD<L, -1, false, Q * z_line_stride8(L), false, Q>;
     using FI = LineFFTDD<L, +1, false, Q * z_line_stride8(L), false, Q>;
     FF::run(v, line_sm, t, tw2);
     if (MUL) {
 #pragma unroll
-        for (int i = 0; i < kE8; ++i) v[i] = cmul(v[i], ok ? cdd_load_nc(K2 + base + (long)(t + TPL * i) * Y) : czero_dd());
+        for (int i = 0; i < kE8; ++i) v[i] = cdp_mul_pair(v[i], ok ? cdp_load_nc(K2 + base + (long)(t + TPL * i) * Y) : cdp_zero());
         __syncthreads();
         FI::run(v, line_sm, t, tw2);
     } else {
 #pragma unroll
-        for (int i = 0; i < kE8; ++i) v[i] = cdd{dd_mul(v[i].re, scale), dd_mul(v[i].im, scale)};
+        for (int i = 0; i < kE8; ++i) v[i] = cdp_scale(v[i], scale);
     }
     if (ok) {
 #pragma unroll
-        for (int i = 0; i < kE8; ++i) cdd_store(S2 + base + (long)(t + TPL * i) * Y, v[i]);
+        for (int i = 0; i < kE8; ++i) cdp_store(S2 + base + (long)(t + TPL * i) * Y, v[i]);
     }
 }
 
@@ -417,13 +421,13 @@ __device__ __forceinline__ void ddf_z2_pipe(cdd* __restrict__ S2, const cdd* __r
     for (; tile < ntiles; tile += gridDim.x) {
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         const long next = tile + gridDim.x;
-        cdd v[kE8];
+        cdp v[kE8];
 #pragma unroll
-        for (int i = 0; i < kE8; ++i) v[i] = stS[i * kDdThreads];
+        for (int i = 0; i < kE8; ++i) v[i] = cdp_load(stS + i * kDdThreads);
         if (next < ntiles) issue(stS, S2, next);
         LineFFTDD<L, -1, false, 0, true, Q>::run(v, line_sm, t, tws);
 #pragma unroll
-        for (int i = 0; i < kE8; ++i) v[i] = cmul_pair(v[i], stK[i * kDdThreads]);
+        for (int i = 0; i < kE8; ++i) v[i] = cdp_mul_pair(v[i], cdp_load(stK + i * kDdThreads));
         if (next < ntiles) issue(stK, K2, next);
         // no barrier here nor at the loop's end: the next transform writes the
         // column lines only after its bound reduction's block barrier, which
@@ -434,7 +438,7 @@ __device__ __forceinline__ void ddf_z2_pipe(cdd* __restrict__ S2, const cdd* __r
         if (ok) {
             cdd* col = S2 + o;
 #pragma unroll
-            for (int i = 0; i < kE8; ++i) cdd_store(col + i * step, v[i]);
+            for (int i = 0; i < kE8; ++i) cdp_store(col + i * step, v[i]);
         }
     }
 }
@@ -454,12 +458,12 @@ struct DdXFast {
 // unpack the packed forward double-float spectra (natural order in registers
 // of pair p) into the two half spectra, coalesced over rows
 template <int L>
-__device__ __forceinline__ void ddf_store_halves(const DdXFast& a, cdd (&v)[kE8], cdd* sm, int p, int t, long rho0,
+__device__ __forceinline__ void ddf_store_halves(const DdXFast& a, cdp (&v)[kE8], cdd* sm, int p, int t, long rho0,
                                                  int nrows) {
     constexpr int TPL = L / kE8, P = ddf_pairs(L), LS = x_line_stride8(L), XH = L / 2 + 1;
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kE8; ++q) cdd_store(sm + p * LS + pad8(t + TPL * q), v[q]);
+    for (int q = 0; q < kE8; ++q) cdp_store(sm + p * LS + pad8(t + TPL * q), v[q]);
     __syncthreads();
     for (int idx = threadIdx.x; idx < XH * 2 * P; idx += kDdThreads) {
         const int k = idx / (2 * P), row = idx - k * 2 * P;
@@ -467,16 +471,10 @@ __device__ __forceinline__ void ddf_store_halves(const DdXFast& a, cdd (&v)[kE8]
         const int pp = row < P ? row : row - P;
         // zk and zm are outputs of one aligned line (one grid, below 2^23 q):
         // their sums and differences are exact FP32 adds
-        const cdd zk = cdd_load(sm + pp * LS + pad8(k));
-        const cdd zm = cconj(cdd_load(sm + pp * LS + pad8(k == 0 ? 0 : L - k)));
-        cdd val;
-        if (row < P) {
-            val = chalf(adf_cadd(zk, zm));
-        } else {
-            const cdd d = chalf(adf_csub(zk, zm));
-            val = cdd{d.im, dd{-d.re.hi, -d.re.lo}};
-        }
-        cdd_store(a.S2 + (long)k * a.YZ + rho0 + row, val);
+        const cdp zk = cdp_load(sm + pp * LS + pad8(k));
+        const cdp zm = cdp_conj(cdp_load(sm + pp * LS + pad8(k == 0 ? 0 : L - k)));
+        const cdp val = row < P ? cdp_add(zk, zm) : cdp_muli<-1>(cdp_sub(zk, zm));
+        cdp_store(a.S2 + (long)k * a.YZ + rho0 + row, cdp_half(val));
     }
 }
 
@@ -489,11 +487,11 @@ __device__ __forceinline__ void ddf_x_forward_tile(const DdXFast& a, long tile, 
     const bool oka = p < nrows, okb = P + p < nrows;
     const float* ra = a.src + (rho0 + p) * L;
     const float* rb = a.src + (rho0 + P + p) * L;
-    cdd v[kE8];
+    cdp v[kE8];
 #pragma unroll
     for (int q = 0; q < kE8; ++q) {
         const int n = t + TPL * q;
-        v[q] = cdd{dd_from(oka ? ld1<CO>(ra + n) : 0.f), dd_from(okb ? ld1<CO>(rb + n) : 0.f)};
+        v[q] = cdp_from(oka ? ld1<CO>(ra + n) : 0.f, okb ? ld1<CO>(rb + n) : 0.f);
     }
     LineFFTDD<L, -1, true>::run(v, sm + p * LS, t, a.tw2, 1 + p);
     ddf_store_halves<L>(a, v, sm, p, t, rho0, nrows);
@@ -514,15 +512,15 @@ __device__ __forceinline__ void ddf_gather_issue(const DdXFast& a, long rho0, in
 
 // the full spectrum of the complex line A + iB of pair p from the gathered halves
 template <int L>
-__device__ __forceinline__ void ddf_pair_line(const cdd* sm, int p, int t, cdd (&v)[kE8]) {
+__device__ __forceinline__ void ddf_pair_line(const cdd* sm, int p, int t, cdp (&v)[kE8]) {
     constexpr int TPL = L / kE8, P = ddf_pairs(L), HS = x_half_stride8(L);
 #pragma unroll
     for (int q = 0; q < kE8; ++q) {
         const int k = t + TPL * q;
         const int kk = k <= L / 2 ? k : L - k;
-        const cdd A = cdd_load(sm + p * HS + kk), B = cdd_load(sm + (P + p) * HS + kk);
-        v[q] = k <= L / 2 ? cdd{dd_sub(A.re, B.im), dd_add(A.im, B.re)}    // A + iB
-                          : cdd{dd_add(A.re, B.im), dd_sub(B.re, A.im)};   // conj(A) + i conj(B)
+        const cdp A = cdp_load(sm + p * HS + kk), B = cdp_muli<+1>(cdp_load(sm + (P + p) * HS + kk));
+        // A + iB, or conj(A) + i conj(B) = conj(A - iB)
+        v[q] = k <= L / 2 ? cdp_two_add(A, B) : cdp_conj(cdp_two_add(A, cdp_neg(B)));
     }
 }
 
@@ -530,7 +528,7 @@ __device__ __forceinline__ void ddf_pair_line(const cdd* sm, int p, int t, cdd (
 // tile and form the full spectrum of the complex line A + iB in v
 template <int L, bool CO>
 __device__ __forceinline__ void ddf_gather_pair(const DdXFast& a, long rho0, int nrows, int p, int t, cdd* sm,
-                                                cdd (&v)[kE8]) {
+                                                cdp (&v)[kE8]) {
     ddf_gather_issue<L>(a, rho0, nrows, sm);
     cp_async_wait_all();
     __syncthreads();
@@ -544,7 +542,7 @@ __device__ __forceinline__ void ddf_x_inverse_tile(const DdXFast& a, long tile, 
     const int p = threadIdx.x / TPL, t = threadIdx.x - p * TPL;
     const long rho0 = tile * 2 * P;
     const int nrows = (int)min((long)2 * P, a.YZ - rho0);
-    cdd v[kE8];
+    cdp v[kE8];
     ddf_gather_pair<L, CO>(a, rho0, nrows, p, t, sm, v);
     __syncthreads();
     LineFFTDD<L, +1, true>::run(v, sm + p * LS, t, a.tw2, 1 + p);
@@ -552,8 +550,9 @@ __device__ __forceinline__ void ddf_x_inverse_tile(const DdXFast& a, long tile, 
 #pragma unroll
     for (int q = 0; q < kE8; ++q) {
         const int n = t + TPL * q;
-        if (p < nrows) a.dst[ra + n] = v[q].re.hi + v[q].re.lo;
-        if (P + p < nrows) a.dst[rb + n] = v[q].im.hi + v[q].im.lo;
+        const float2 z = cdp_round(v[q]);
+        if (p < nrows) a.dst[ra + n] = z.x;
+        if (P + p < nrows) a.dst[rb + n] = z.y;
     }
 }
 
@@ -586,7 +585,7 @@ __device__ __forceinline__ void ddf_x_ratio_tile(const DdXFast& a, long tile, cd
     }
     cp_async_wait_all();
     __syncthreads();
-    cdd v[kE8];
+    cdp v[kE8];
     ddf_pair_line<L>(sm, p, t, v);
     __syncthreads();
     LineFFTDD<L, +1, true>::run(v, sm + p * LS, t, a.tw2, 1 + p);
@@ -602,7 +601,8 @@ __device__ __forceinline__ void ddf_x_ratio_tile(const DdXFast& a, long tile, cd
         // exact where phi and b' are within a factor 2 (Sterbenz), so r - 1
         // keeps its relative precision as r approaches 1; the quotient is the
         // fast division intrinsic (2 ulp, b' far inside its range)
-        const float ba = fmaxf(v[q].re.hi + v[q].re.lo, a.eps), bb = fmaxf(v[q].im.hi + v[q].im.lo, a.eps);
+        const float2 z = cdp_round(v[q]);
+        const float ba = fmaxf(z.x, a.eps), bb = fmaxf(z.y, a.eps);
         const float xa = oka ? __fdividef(phs[p * L + n] - ba, ba) : 0.f;
         const float xb = okb ? __fdividef(phs[(P + p) * L + n] - bb, bb) : 0.f;
         f[q] = make_float2(xa, xb);
@@ -631,7 +631,7 @@ __device__ __forceinline__ void ddf_x_ratio_tile(const DdXFast& a, long tile, cd
         if (a.S)
             a.S[(long)k * a.YZ + rho0 + row] = val;
         else
-            cdd_store(a.S2 + (long)k * a.YZ + rho0 + row, cdd{dd_from(val.x), dd_from(val.y)});
+            cdp_store(a.S2 + (long)k * a.YZ + rho0 + row, cdp_from(val.x, val.y));
     }
 }
 
@@ -674,7 +674,7 @@ __device__ __forceinline__ void ddf_x_update_tile(const DdXUpd& a, long tile, cd
     }
     cp_async_wait_all();
     __syncthreads();
-    cdd v[kE8];
+    cdp v[kE8];
     ddf_pair_line<L>(sm, p, t, v);
     __syncthreads();
     LineFFTDD<L, +1, true>::run(v, sm + p * LS, t, a.tw2, 1 + p);
@@ -682,7 +682,8 @@ __device__ __forceinline__ void ddf_x_update_tile(const DdXUpd& a, long tile, cd
 #pragma unroll
     for (int q = 0; q < kE8; ++q) {
         const int n = t + TPL * q;
-        const float ca = v[q].re.hi + v[q].re.lo, cb = v[q].im.hi + v[q].im.lo;  // c - 1
+        const float2 z = cdp_round(v[q]);
+        const float ca = z.x, cb = z.y;  // c - 1
         const float pa = ps[p * L + n], pb = ps[(P + p) * L + n];
         if (MODE == 1) {
             if (oka) a.psi[ra + n] = fmaxf(pa * update_factor(ca, pa, a.wt, ra + n, a.lam, a.inv_s), a.eps);

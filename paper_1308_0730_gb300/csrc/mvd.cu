@@ -363,7 +363,7 @@ mvd_status setup_fft(mvd_ctx* c) {
             const double ang = -2.0 * M_PI * (double)m / (double)L;
             const double cr = std::cos(ang), ci = std::sin(ang);
             const float rh = (float)cr, ih = (float)ci;
-            return make_float4(rh, (float)(cr - rh), ih, (float)(ci - ih));
+            return make_float4(rh, ih, (float)(cr - rh), (float)(ci - ih));  // the order of adp.cuh
         };
         std::vector<float4> tw2(3 * ((size_t)g.X + g.Y + g.Z), make_float4(0.f, 0.f, 0.f, 0.f));
         size_t o = 0;
