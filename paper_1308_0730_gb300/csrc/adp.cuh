@@ -253,4 +253,46 @@ struct DftP<5, S> {
     }
 };
 
+// length 6 as 2 x 3 with coprime factors (Good-Thomas): no twiddles between
+template <int S>
+struct DftP<6, S> {
+    __device__ __forceinline__ static void run(cdp* v, f2 c) {
+        cdp a[3] = {cdp_add(v[0], v[3]), cdp_add(v[2], v[5]), cdp_add(v[4], v[1])};
+        cdp b[3] = {cdp_sub(v[0], v[3]), cdp_sub(v[2], v[5]), cdp_sub(v[4], v[1])};
+        DftP<3, S>::run(a, c);
+        DftP<3, S>::run(b, c);
+        v[0] = a[0], v[4] = a[1], v[2] = a[2];
+        v[3] = b[0], v[1] = b[1], v[5] = b[2];
+    }
+};
+
+// length 9 as 3 x 3 with the internal twiddles exp(s 2 pi i m / 9), m = 1, 2, 4
+template <int S>
+struct DftP<9, S> {
+    __device__ __forceinline__ static cdp mul_root(cdp x, int m, f2 c) {
+        const double cr = m == 1 ? 0.76604444311897803520 : m == 2 ? 0.17364817766693034885 : -0.93969262078590838405;
+        const double si = m == 1 ? 0.64278760968653932632 : m == 2 ? 0.98480775301220805936 : 0.34202014332566873304;
+        const dd r = MVD_DD(cr), i = MVD_DD(S * si);
+        const cdp xs{f2_swap(x.h), f2_swap(x.l)};
+        return cdp_add(cdp_mulk(x, r, c), cdp_mulk(xs, f2_of(-i.hi, i.hi), f2_of(-i.lo, i.lo), c));
+    }
+    __device__ __forceinline__ static void run(cdp* v, f2 c) {
+        cdp c0[3] = {v[0], v[3], v[6]};
+        cdp c1[3] = {v[1], v[4], v[7]};
+        cdp c2[3] = {v[2], v[5], v[8]};
+        DftP<3, S>::run(c0, c);
+        DftP<3, S>::run(c1, c);
+        DftP<3, S>::run(c2, c);
+        cdp r0[3] = {c0[0], c1[0], c2[0]};
+        cdp r1[3] = {c0[1], mul_root(c1[1], 1, c), mul_root(c2[1], 2, c)};
+        cdp r2[3] = {c0[2], mul_root(c1[2], 2, c), mul_root(c2[2], 4, c)};
+        DftP<3, S>::run(r0, c);
+        DftP<3, S>::run(r1, c);
+        DftP<3, S>::run(r2, c);
+        v[0] = r0[0], v[3] = r0[1], v[6] = r0[2];
+        v[1] = r1[0], v[4] = r1[1], v[7] = r1[2];
+        v[2] = r2[0], v[5] = r2[1], v[8] = r2[2];
+    }
+};
+
 }  // namespace mvd

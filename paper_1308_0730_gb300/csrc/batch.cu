@@ -97,7 +97,7 @@ __device__ __forceinline__ void with_len(int L, F&& f) {
 
 // precise mode, axes of length 64, 128 or 256: register-resident
 // double-float passes (the same tiles as the single-volume engine)
-__device__ bool run_tile_ddf(const VolDesc& d, int pass, int view, long tile, cdd* sm) {
+__device__ __noinline__ bool run_tile_ddf(const VolDesc& d, int pass, int view, long tile, cdd* sm) {
     const size_t ns = (size_t)d.Xh * d.YZ;
     switch (pass) {
         case XF:
@@ -141,8 +141,26 @@ __device__ bool run_tile_ddf(const VolDesc& d, int pass, int view, long tile, cd
     }
 }
 
+// The mixed-radix tiles as functions of their own: inlined together they make one
+// function that takes minutes to compile.
+#define MVD_TILE_FN(NAME, ARGS, ELEM, CALL) \
+    __device__ __noinline__ void NAME(const ARGS& a, long tile, ELEM* sm) { CALL; }
+MVD_TILE_FN(t_dd_xf, DdX, cdd, dd_x_forward_tile<true>(a, tile, sm))
+MVD_TILE_FN(t_dd_xr, DdX, cdd, dd_x_ratio_tile<true>(a, tile, sm))
+MVD_TILE_FN(t_dd_yf, DdY, cdd, (dd_y_tile<true, -1>(a, tile, sm)))
+MVD_TILE_FN(t_dd_yi, DdY, cdd, (dd_y_tile<true, +1>(a, tile, sm)))
+MVD_TILE_FN(t_dd_z, DdZ, cdd, (dd_z_tile<true, true>(a, tile, sm)))
+MVD_TILE_FN(t_dd_xu, DdXU, cdd, (dd_x_update_tile<true, 1>(a, tile, sm)))
+MVD_TILE_FN(t_xf, GenX, float2, gen_x_forward_tile<true>(a, tile, sm))
+MVD_TILE_FN(t_xr, GenX, float2, gen_x_ratio_tile<true>(a, tile, sm))
+MVD_TILE_FN(t_yf, GenY, float2, (gen_y_tile<true, -1>(a, tile, sm)))
+MVD_TILE_FN(t_yi, GenY, float2, (gen_y_tile<true, +1>(a, tile, sm)))
+MVD_TILE_FN(t_z, GenZ, float2, (gen_z_tile<true, true>(a, tile, sm)))
+MVD_TILE_FN(t_xu, GenX, float2, (gen_x_inverse_tile<true, 1>(a, tile, sm)))
+#undef MVD_TILE_FN
+
 // precise mode: every pass but the update runs in double-float
-__device__ void run_tile_dd(const VolDesc& d, int pass, int view, long tile, cdd* sm) {
+__device__ __noinline__ void run_tile_dd(const VolDesc& d, int pass, int view, long tile, cdd* sm) {
     const size_t ns = (size_t)d.Xh * d.YZ;
     if (run_tile_ddf(d, pass, view, tile, sm)) return;
     switch (pass) {
@@ -150,22 +168,22 @@ __device__ void run_tile_dd(const VolDesc& d, int pass, int view, long tile, cdd
             DdX a = dd_x_args(d.X, d.YZ, d.px, d.tw2x);
             a.src = d.psi;
             a.S2 = d.S2;
-            dd_x_forward_tile<true>(a, tile, sm);
+            t_dd_xf(a, tile, sm);
             break;
         }
         case YF1:
         case YF2:
-            dd_y_tile<true, -1>(dd_y_args(d.Y, d.Xh, d.Z, d.py, d.tw2y, d.S2), tile, sm);
+            t_dd_yf(dd_y_args(d.Xh, d.Z, d.py, d.tw2y, d.S2), tile, sm);
             break;
         case YI1:
         case YI2:
-            dd_y_tile<true, +1>(dd_y_args(d.Y, d.Xh, d.Z, d.py, d.tw2y, d.S2), tile, sm);
+            t_dd_yi(dd_y_args(d.Xh, d.Z, d.py, d.tw2y, d.S2), tile, sm);
             break;
         case Z1:
         case Z2: {
             const cdd* K2 = reinterpret_cast<const cdd*>(reinterpret_cast<const float4*>(d.KP2) +
                                                          ns * (2 * view + (pass == Z2 ? 1 : 0)));
-            dd_z_tile<true, true>(dd_z_args(d.Z, d.Y, d.YZ, d.pz, d.tw2z, d.S2, K2, dd{1.f, 0.f}), tile, sm);
+            t_dd_z(dd_z_args(d.Y, d.YZ, d.pz, d.tw2z, d.S2, K2, dd{1.f, 0.f}), tile, sm);
             break;
         }
         default: {  // XR
@@ -173,13 +191,13 @@ __device__ void run_tile_dd(const VolDesc& d, int pass, int view, long tile, cdd
             a.S2 = d.S2;
             a.phi = d.views + (size_t)view * d.M;
             a.eps = d.eps;
-            dd_x_ratio_tile<true>(a, tile, sm);
+            t_dd_xr(a, tile, sm);
             break;
         }
     }
 }
 
-__device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2* sm) {
+__device__ __noinline__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2* sm) {
     const size_t ns = (size_t)d.Xh * d.YZ;
     if (d.precise && pass != XU) {
         run_tile_dd(d, pass, view, tile, reinterpret_cast<cdd*>(sm));
@@ -194,7 +212,7 @@ __device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2
                 GenX a = gen_x_args(d.X, d.YZ, d.px);
                 a.src = d.psi;
                 a.S = d.S;
-                gen_x_forward_tile<true>(a, tile, sm);
+                t_xf(a, tile, sm);
             }
             break;
         }
@@ -213,9 +231,9 @@ __device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2
                         fast_y_tile<L, -1, true>(d.S, nl, d.py.tw, tile, sm);
                 });
             } else if (inv) {
-                gen_y_tile<true, +1>(gen_y_args(d.Y, d.Xh, d.Z, d.py, d.S), tile, sm);
+                t_yi(gen_y_args(d.Xh, d.Z, d.py, d.S), tile, sm);
             } else {
-                gen_y_tile<true, -1>(gen_y_args(d.Y, d.Xh, d.Z, d.py, d.S), tile, sm);
+                t_yf(gen_y_args(d.Xh, d.Z, d.py, d.S), tile, sm);
             }
             break;
         }
@@ -229,7 +247,7 @@ __device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2
                     fast_z_tile<L, true, true>(d.S, K, d.Y, d.YZ, nty, 1.f, d.pz.tw, tile, sm);
                 });
             } else {
-                gen_z_tile<true, true>(gen_z_args(d.Z, d.Y, d.YZ, d.pz, d.S, K, 1.f), tile, sm);
+                t_z(gen_z_args(d.Y, d.YZ, d.pz, d.S, K, 1.f), tile, sm);
             }
             break;
         }
@@ -242,7 +260,7 @@ __device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2
                 a.S = d.S;
                 a.phi = d.views + (size_t)view * d.M;
                 a.eps = d.eps;
-                gen_x_ratio_tile<true>(a, tile, sm);
+                t_xr(a, tile, sm);
             }
             break;
         }
@@ -259,7 +277,7 @@ __device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2
                     u.x.S2 = d.S2;
                     u.x.eps = d.eps;
                     u.psi = d.psi;
-                    dd_x_update_tile<true, 1>(u, tile, reinterpret_cast<cdd*>(sm));
+                    t_dd_xu(u, tile, reinterpret_cast<cdd*>(sm));
                 }
             } else if (d.fx) {
                 const XFast a{nullptr, d.S, nullptr, d.psi, d.YZ, d.eps, d.px.tw};
@@ -269,7 +287,7 @@ __device__ void run_tile(const VolDesc& d, int pass, int view, long tile, float2
                 a.S = d.S;
                 a.psi = d.psi;
                 a.eps = d.eps;
-                gen_x_inverse_tile<true, 1>(a, tile, sm);
+                t_xu(a, tile, sm);
             }
             break;
         }
@@ -336,8 +354,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                     *elems = 2L * ddf_pairs(d.X) * d.X * 4;
                     return;
                 }
-                *ntiles = dd_x_tiles(d.X, d.YZ);
-                *elems = 2L * dd_x_pairs(d.X) * d.X * 4;  // double-float work counts about 4x
+                *ntiles = dd_x_tiles(d.px, d.YZ);
+                *elems = 2L * dd_x_geo(d.px).n() * d.X * 4;  // double-float work counts about 4x
                 return;
             case Z1:
             case Z2:
@@ -346,8 +364,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                     *elems = (long)ddf_z_cols(d.Z) * d.Z * 4;
                     return;
                 }
-                *ntiles = dd_z_tiles(d.Z, d.Y, d.Xh);
-                *elems = (long)dd_z_cols(d.Z, d.Y) * d.Z * 4;
+                *ntiles = dd_z_tiles(d.pz, d.Y, d.Xh);
+                *elems = (long)dd_line_geo(d.pz, d.Y).n() * d.Z * 4;
                 return;
             default:
                 if (d.fy) {
@@ -355,8 +373,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                     *elems = (long)ddf_y_lines(d.Y) * d.Y * 4;
                     return;
                 }
-                *ntiles = dd_y_tiles(d.Y, d.Xh, d.Z);
-                *elems = (long)dd_y_lines(d.Y) * d.Y * 4;
+                *ntiles = dd_y_tiles(d.py, d.Xh, d.Z);
+                *elems = (long)dd_line_geo(d.py, 32).n() * d.Y * 4;
                 return;
         }
     }
@@ -368,8 +386,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                 *ntiles = gen_div_up(d.YZ, fast_x_rows(d.X));
                 *elems = (long)fast_x_rows(d.X) * d.X;
             } else {
-                *ntiles = gen_x_tiles(d.X, d.YZ);
-                *elems = 2L * gen_x_pairs(d.X) * d.X;
+                *ntiles = gen_x_tiles(d.px, d.YZ);
+                *elems = 2L * gen_x_geo(d.px).n() * d.X;
             }
             return;
         case Z1:
@@ -378,8 +396,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                 *ntiles = (long)d.Xh * gen_div_up(d.Y, fast_z_cols(d.Z));
                 *elems = (long)fast_z_cols(d.Z) * d.Z;
             } else {
-                *ntiles = gen_z_tiles(d.Z, d.Y, d.Xh);
-                *elems = (long)gen_z_cols(d.Z, d.Y) * d.Z;
+                *ntiles = gen_z_tiles(d.pz, d.Y, d.Xh);
+                *elems = (long)gen_line_geo(d.pz, d.Y).n() * d.Z;
             }
             return;
         default:
@@ -387,8 +405,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                 *ntiles = gen_div_up((long)d.Xh * d.Z, fast_y_lines(d.Y));
                 *elems = (long)fast_y_lines(d.Y) * d.Y;
             } else {
-                *ntiles = gen_y_tiles(d.Y, d.Xh, d.Z);
-                *elems = (long)gen_y_lines(d.Y) * d.Y;
+                *ntiles = gen_y_tiles(d.py, d.Xh, d.Z);
+                *elems = (long)gen_line_geo(d.py, 32).n() * d.Y;
             }
             return;
     }
@@ -612,11 +630,11 @@ mvd_status mvd_batch_create_mode(mvd_ctx* const* ctxs, int n, int n_iter, int mo
         d.tw2x = g.tw2x;
         d.tw2y = g.tw2y;
         d.tw2z = g.tw2z;
-        smem = std::max({smem, d.fx ? fast_x_smem(g.X) : gen_x_smem(g.X), d.fy ? fast_y_smem(g.Y) : gen_y_smem(g.Y),
-                         d.fz ? fast_z_smem(g.Z) : gen_z_smem(g.Z, g.Y)});
+        smem = std::max({smem, d.fx ? fast_x_smem(g.X) : gen_smem(gen_x_geo(g.px)), d.fy ? fast_y_smem(g.Y) : gen_smem(gen_line_geo(g.py, 32)),
+                         d.fz ? fast_z_smem(g.Z) : gen_smem(gen_line_geo(g.pz, g.Y))});
         if (d.precise)
-            smem = std::max({smem, d.fx ? ddf_ratio_smem(g.X) : dd_x_smem(g.X), d.fy ? ddf_y_smem(g.Y) : dd_y_smem(g.Y),
-                             d.fz ? ddf_z_smem(g.Z) : dd_z_smem(g.Z, g.Y)});
+            smem = std::max({smem, d.fx ? ddf_ratio_smem(g.X) : dd_smem(dd_x_geo(g.px)), d.fy ? ddf_y_smem(g.Y) : dd_smem(dd_line_geo(g.py, 32)),
+                             d.fz ? ddf_z_smem(g.Z) : dd_smem(dd_line_geo(g.pz, g.Y))});
     }
     // Entries (default schedule: views 0..nv-1 per iteration). Each volume's
     // own entries stay in order; across volumes they are merged by the

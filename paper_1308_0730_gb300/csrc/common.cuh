@@ -115,9 +115,8 @@ mvd_status fft_x_accumulate_fast(const FftGeom& g, const float2* S, float* acc, 
 // double-float forward blur (fft_dd.cu): spectrum of complex double-float
 mvd_status dd_forward_real(const FftGeom& g, const float* src, cdd* S2, cudaStream_t st);
 mvd_status dd_y(const FftGeom& g, cdd* S2, int inverse, cudaStream_t st);
-// register-resident x and y lengths: the back-projection's forward y pass can
-// take the ratio pass's FP32 spectrum of r - 1 (exact FP32 values) into S2
-bool dd_fast_yx(const FftGeom& g);
+// the back-projection's forward y pass takes the ratio pass's FP32 spectrum of
+// r - 1 (exact FP32 values) into S2
 mvd_status dd_y_from_f32(const FftGeom& g, const float2* S1, cdd* S2, cudaStream_t st);
 // the double-float x inverse of S2 to real rows (rounded to FP32), generic lengths
 mvd_status dd_x_inverse_real_generic(const FftGeom& g, const cdd* S2, float* dst, cudaStream_t st);
@@ -127,6 +126,14 @@ mvd_status dd_x_update(const FftGeom& g, const cdd* S2, float* psi, float eps, c
                        float lam, const float* inv_s, int accumulate);
 mvd_status dd_x_update_generic(const FftGeom& g, const cdd* S2, float* psi, float eps, cudaStream_t st,
                                const float* wt, float lam, const float* inv_s, int accumulate);
+
+// the same passes for lengths without a register-resident form (fft_dd_gen.cu);
+// dd_y_generic: forward from the FP32 spectrum S1 when given; dd_z_generic: without
+// K2 forward, times the scale
+mvd_status dd_forward_real_generic(const FftGeom& g, const float* src, cdd* S2, cudaStream_t st);
+mvd_status dd_x_ratio_generic(const FftGeom& g, cdd* S2, const float* phi, float eps, cudaStream_t st, float2* S);
+mvd_status dd_y_generic(const FftGeom& g, cdd* S2, int inverse, const float2* S1, cudaStream_t st);
+mvd_status dd_z_generic(const FftGeom& g, cdd* S2, const cdd* K2, double scale, cudaStream_t st);
 
 mvd_status dd_z_mul(const FftGeom& g, cdd* S2, const cdd* K2, cudaStream_t st);
 mvd_status dd_z_forward_scaled(const FftGeom& g, cdd* S2, double scale, cudaStream_t st);

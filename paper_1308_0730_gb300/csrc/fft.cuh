@@ -1,6 +1,4 @@
-// Device-side FFT building blocks: complex helpers, radix-2/3/4/5/8 DFT
-// butterflies and a shared-memory Stockham (self-sorting) driver that runs
-// the same length-L transform on a batch of lines held in shared memory.
+// Device-side FFT building blocks: complex helpers and small DFT butterflies.
 //
 // Stockham stage with radix R after Ns points have been combined (Ns starts
 // at 1 and is multiplied by R after each stage): for butterfly j in [0, L/R)
@@ -224,91 +222,11 @@ struct Dft<9, S> {
     __device__ __forceinline__ static void run(float2* v) { dft9<mvd::Dft, S>(v); }
 };
 
-// ---------------------------------------------------------------------------
-// one Stockham butterfly (see the file header)
-// ---------------------------------------------------------------------------
-
 // floor(n / d) for 0 <= n and n + d < 2^22, from inv = the FP32 reciprocal of d
 // (correctly rounded): (n + 1/2) / d lies at least 1/(2d) from an integer and
 // the two roundings move it by less than (n/d + 1) 2^-23, so the truncation is
 // exact. Replaces the integer divisions of the butterfly indexing.
 __device__ __forceinline__ int small_div(int n, float inv) { return __float2int_rz(((float)n + 0.5f) * inv); }
-
-// Per-stage constants of the Stockham indexing: nb = L / R butterflies per
-// line, Ns combined so far.
-struct StageIdx {
-    int nb, Ns;
-    float inv_nb, inv_ns;
-    __device__ __forceinline__ StageIdx(int L, int R, int ns)
-        : nb(L / R), Ns(ns), inv_nb(1.0f / (float)(L / R)), inv_ns(1.0f / (float)ns) {}
-};
-
-template <int R, int S>
-__device__ __forceinline__ void stockham_bfly(const float2* __restrict__ A, float2* __restrict__ B, int j,
-                                              const StageIdx& si, const float2* __restrict__ tw) {
-    const int jq = small_div(j, si.inv_ns);
-    const int k = j - jq * si.Ns;
-    float2 v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = A[j + r * si.nb];
-    if (si.Ns > 1) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = cmul(v[r], twiddle<S>(tw, (r - 1) * si.Ns + k));
-    }
-    Dft<R, S>::run(v);
-    const int d = jq * si.Ns * R + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) B[d + r * si.Ns] = v[r];
-}
-
-// All butterflies of one stage (radix R, Ns combined so far) over `nlines`
-// lines, spread over the block's threads.
-template <int R, int S>
-__device__ __forceinline__ void stockham_stage(const float2* __restrict__ A, float2* __restrict__ B, int nlines,
-                                               int ls, int L, int Ns, const float2* __restrict__ tw) {
-    const StageIdx si(L, R, Ns);
-    const int total = nlines * si.nb;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int line = small_div(t, si.inv_nb);
-        const int j = t - line * si.nb;
-        stockham_bfly<R, S>(A + line * ls, B + line * ls, j, si, tw);
-    }
-}
-
-// Transforms `nlines` lines of length p.L stored at A + line*ls (line stride
-// ls >= L), using B (same shape) as the ping-pong buffer. All threads of the
-// block take part; the call begins and ends with the data synchronised.
-// Returns the buffer (A or B) that holds the result.
-// Twiddles: p.tw is the axis's natural table (w^m, m < L), followed by its
-// radix-8 and radix-16 stage-ordered copies and then by its copy in the
-// stage order of this plan (p.tw + 3L): stage s >= 1 (Ns combined before it,
-// radix R) keeps w^(r k L / (Ns R)) at (earlier stages' entries) +
-// (r - 1) Ns + k, so consecutive butterflies read consecutive entries.
-template <int S>
-__device__ float2* fft_lines(float2* A, float2* B, int nlines, int ls, const FftPlan& p) {
-    int Ns = 1;
-    const float2* tw = p.tw + 3 * p.L;
-    for (int s = 0; s < p.nst; ++s) {
-        const int R = p.radix[s];
-        switch (R) {
-            case 8: stockham_stage<8, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            case 4: stockham_stage<4, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            case 2: stockham_stage<2, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            case 3: stockham_stage<3, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            case 6: stockham_stage<6, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            case 9: stockham_stage<9, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            case 10: stockham_stage<10, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-            default: stockham_stage<5, S>(A, B, nlines, ls, p.L, Ns, tw); break;
-        }
-        if (s > 0) tw += (R - 1) * Ns;
-        __syncthreads();
-        float2* t = A;
-        A = B;
-        B = t;
-        Ns *= R;
-    }
-    return A;
-}
 
 // Global loads of data that other blocks of the same launch may have written
 // (the persistent batch kernel) must bypass L1: CO selects L2-only loads.

@@ -1,46 +1,12 @@
-// Kernels and launchers of the double-float forward-blur passes (tile
-// functions in fft_dd.cuh).
+// Kernels and launchers of the register-resident double-float passes (tile
+// functions in fft_dd_fast.cuh); other lengths go to fft_dd_gen.cu.
 #include <type_traits>
 
-#include "fft_dd.cuh"
 #include "fft_dd_fast.cuh"
 
 namespace mvd {
 
 namespace {
-
-// generic double-float passes: three blocks per SM (their tiles' shared
-// memory allows three; the registers of the radix-9/10 butterflies would
-// otherwise leave room for two)
-constexpr int kDdGenBlocks = 3;
-
-__global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_forward(DdX a) {
-    extern __shared__ cdd smd[];
-    dd_x_forward_tile<false>(a, blockIdx.x, smd);
-}
-
-__global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_ratio(DdX a) {
-    extern __shared__ cdd smd[];
-    dd_x_ratio_tile<false>(a, blockIdx.x, smd);
-}
-
-template <int MODE>
-__global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_update(DdXU u) {
-    extern __shared__ cdd smd[];
-    dd_x_update_tile<false, MODE>(u, blockIdx.x, smd);
-}
-
-template <int S>
-__global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_y(DdY a) {
-    extern __shared__ cdd smd[];
-    dd_y_tile<false, S>(a, blockIdx.x, smd);
-}
-
-template <bool MUL>
-__global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_z(DdZ a) {
-    extern __shared__ cdd smd[];
-    dd_z_tile<false, MUL>(a, blockIdx.x, smd);
-}
 
 // register-resident double-float passes (power-of-two lengths)
 template <int L, int S, int IO = 0>
@@ -138,17 +104,6 @@ DdXFast ddf_args(const FftGeom& g) {
     return a;
 }
 
-template <typename K, typename A>
-mvd_status launch(K kern, const A& a, long grid, size_t smem, cudaStream_t st, const char* name, int cls) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_status(e, name);
-    prof_begin(cls, st);
-    kern<<<(unsigned)grid, kGenThreads, smem, st>>>(a);
-    prof_end(cls, st);
-    count_launch();
-    return check_launch(name);
-}
-
 }  // namespace
 
 mvd_status dd_forward_real(const FftGeom& g, const float* src, cdd* S2, cudaStream_t st) {
@@ -164,10 +119,7 @@ mvd_status dd_forward_real(const FftGeom& g, const float* src, cdd* S2, cudaStre
         });
         return rc;
     }
-    DdX a = dd_x_args(g.X, g.YZ, g.px, g.tw2x);
-    a.src = src;
-    a.S2 = S2;
-    return launch(k_dd_x_forward, a, dd_x_tiles(g.X, g.YZ), dd_x_smem(g.X), st, "dd x forward", KC_DD_X_FORWARD);
+    return dd_forward_real_generic(g, src, S2, st);
 }
 
 bool dd_fast_x(const FftGeom& g) { return g.fast && dd_fast_length(g.X); }
@@ -204,12 +156,7 @@ mvd_status dd_x_ratio(const FftGeom& g, cdd* S2, const float* phi, float eps, cu
         });
         return rc;
     }
-    DdX a = dd_x_args(g.X, g.YZ, g.px, g.tw2x);
-    a.S2 = S2;
-    a.S = S;
-    a.phi = phi;
-    a.eps = eps;
-    return launch(k_dd_x_ratio, a, dd_x_tiles(g.X, g.YZ), dd_x_smem(g.X), st, "dd x ratio", KC_DD_X_RATIO);
+    return dd_x_ratio_generic(g, S2, phi, eps, st, S);
 }
 
 mvd_status dd_y(const FftGeom& g, cdd* S2, int inverse, cudaStream_t st) {
@@ -223,18 +170,11 @@ mvd_status dd_y(const FftGeom& g, cdd* S2, int inverse, cudaStream_t st) {
         });
         return rc;
     }
-    DdY a = dd_y_args(g.Y, g.Xh, g.Z, g.py, g.tw2y, S2);
-    return launch(inverse ? k_dd_y<+1> : k_dd_y<-1>, a, dd_y_tiles(g.Y, g.Xh, g.Z), dd_y_smem(g.Y), st, "dd y",
-                  KC_DD_Y);
+    return dd_y_generic(g, S2, inverse, nullptr, st);
 }
 
-bool dd_fast_yx(const FftGeom& g) { return g.fast && dd_fast_length(g.X) && dd_fast_length(g.Y); }
-
 mvd_status dd_y_from_f32(const FftGeom& g, const float2* S1, cdd* S2, cudaStream_t st) {
-    if (!dd_fast_yx(g)) {
-        set_error("dd y from FP32: needs register-resident x and y lengths, got %d x %d", g.X, g.Y);
-        return MVD_ERR_UNSUPPORTED;
-    }
+    if (!(g.fast && dd_fast_length(g.Y))) return dd_y_generic(g, S2, 0, S1, st);
     mvd_status rc = MVD_ERR_UNSUPPORTED;
     const long nl = (long)g.Xh * g.Z;
     with_dd_len(g.Y, [&](auto Lc) {
@@ -243,28 +183,6 @@ mvd_status dd_y_from_f32(const FftGeom& g, const float2* S1, cdd* S2, cudaStream
                         "dd y (FP32 in)", KC_DD_Y, S2, nl, g.tw2y, const_cast<float2*>(S1));
     });
     return rc;
-}
-
-mvd_status dd_x_update_generic(const FftGeom& g, const cdd* S2, float* psi, float eps, cudaStream_t st,
-                               const float* wt, float lam, const float* inv_s, int accumulate) {
-    DdXU u{};
-    u.x = dd_x_args(g.X, g.YZ, g.px, g.tw2x);
-    u.x.S2 = const_cast<cdd*>(S2);
-    u.x.eps = eps;
-    u.psi = psi;
-    u.wt = wt;
-    u.lam = lam;
-    u.inv_s = inv_s;
-    return launch(accumulate ? k_dd_x_update<4> : k_dd_x_update<1>, u, dd_x_tiles(g.X, g.YZ), dd_x_smem(g.X), st,
-                  "dd x update", KC_X_UPDATE);
-}
-
-mvd_status dd_x_inverse_real_generic(const FftGeom& g, const cdd* S2, float* dst, cudaStream_t st) {
-    DdXU u{};
-    u.x = dd_x_args(g.X, g.YZ, g.px, g.tw2x);
-    u.x.S2 = const_cast<cdd*>(S2);
-    u.psi = dst;
-    return launch(k_dd_x_update<0>, u, dd_x_tiles(g.X, g.YZ), dd_x_smem(g.X), st, "dd x inverse", KC_X_UPDATE);
 }
 
 mvd_status dd_x_update(const FftGeom& g, const cdd* S2, float* psi, float eps, cudaStream_t st, const float* wt,
@@ -310,15 +228,13 @@ mvd_status dd_z_mul(const FftGeom& g, cdd* S2, const cdd* K2, cudaStream_t st) {
         return rc;
     }
     if (g.fast && dd_fast_length(g.Z)) return ddf_z(g, S2, K2, dd{1.f, 0.f}, true, st);
-    DdZ a = dd_z_args(g.Z, g.Y, g.YZ, g.pz, g.tw2z, S2, K2, dd{1.f, 0.f});
-    return launch(k_dd_z<true>, a, dd_z_tiles(g.Z, g.Y, g.Xh), dd_z_smem(g.Z, g.Y), st, "dd z", KC_DD_Z_MUL);
+    return dd_z_generic(g, S2, K2, 1.0, st);
 }
 
 mvd_status dd_z_forward_scaled(const FftGeom& g, cdd* S2, double scale, cudaStream_t st) {
     const float hi = (float)scale;
     if (g.fast && dd_fast_length(g.Z)) return ddf_z(g, S2, nullptr, dd{hi, (float)(scale - (double)hi)}, false, st);
-    DdZ a = dd_z_args(g.Z, g.Y, g.YZ, g.pz, g.tw2z, S2, nullptr, dd{hi, (float)(scale - (double)hi)});
-    return launch(k_dd_z<false>, a, dd_z_tiles(g.Z, g.Y, g.Xh), dd_z_smem(g.Z, g.Y), st, "dd z forward", KC_SETUP);
+    return dd_z_generic(g, S2, nullptr, scale, st);
 }
 
 }  // namespace mvd

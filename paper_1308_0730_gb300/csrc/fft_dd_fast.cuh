@@ -8,6 +8,7 @@
 #include "adf.cuh"
 #include "adp.cuh"
 #include "dd.cuh"
+#include "fft_dd.cuh"
 #include "fft_fast.cuh"
 
 namespace mvd {
@@ -288,14 +289,6 @@ __host__ __device__ constexpr size_t ddf_y_smem(int L) { return (size_t)ddf_y_li
 __host__ __device__ constexpr int z_line_stride8(int L) { return L + L / 8 + (ddf_z_cols(L) == 4 ? 2 : 1); }
 __host__ __device__ constexpr size_t ddf_z_smem(int L) {
     return (size_t)2 * ddf_z_cols(L) * z_line_stride8(L) * sizeof(cdd);
-}
-
-template <bool CO>
-__device__ __forceinline__ cdp ld_cdp(const cdd* p) {
-    if constexpr (CO)
-        return cdp_load_cg(p);
-    else
-        return cdp_load(p);
 }
 
 // IO selects where the lines come from:

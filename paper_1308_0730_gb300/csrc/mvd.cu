@@ -566,20 +566,15 @@ mvd_status mvd::view_pass(mvd_ctx* c, int v, float* prod) {
             // in double-float, so no rounding of a large |r - 1| (a count where
             // b is near eps) spreads over the volume at FP32 level.
             const cdd* Kc2 = reinterpret_cast<const cdd*>(K4 + ns * (2 * v + 1));
-            // The ratio pass hands r - 1 over as an FP32 spectrum when the
-            // forward y pass can widen it (exact FP32 values, half the bytes);
+            // The ratio pass hands r - 1 over as an FP32 spectrum, which the
+            // forward y pass widens (exact FP32 values, half the bytes);
             // every transform after it runs in double-float, the update's x
             // inverse included: an FP32 x inverse there carries the rounding
             // of a line's large values (where b is near eps) into the whole
             // line and left up to 1.4e-4 after 15 iterations on volumes of
             // the 48-volume batch (double-float: <= 2.6e-5).
-            if (dd_fast_yx(g)) {
-                MVD_TRY(dd_x_ratio(g, S2, phi, c->eps, c->stream, c->d_S));
-                MVD_TRY(dd_y_from_f32(g, c->d_S, S2, c->stream));
-            } else {
-                MVD_TRY(dd_x_ratio(g, S2, phi, c->eps, c->stream));
-                MVD_TRY(dd_y(g, S2, 0, c->stream));
-            }
+            MVD_TRY(dd_x_ratio(g, S2, phi, c->eps, c->stream, c->d_S));
+            MVD_TRY(dd_y_from_f32(g, c->d_S, S2, c->stream));
             MVD_TRY(dd_z_mul(g, S2, Kc2, c->stream));
             MVD_TRY(dd_y(g, S2, 1, c->stream));
             if (mirror) {
