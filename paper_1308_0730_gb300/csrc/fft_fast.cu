@@ -40,8 +40,13 @@ __global__ void __launch_bounds__(kThreads) k_x_forward_fast(XFast a) {
     fast_x_forward_tile<L, false>(a, blockIdx.x, sm);
 }
 
-template <int L, int MODE>  // MODE 0: ratio -> forward ; 1: psi update ; 2: plain real output
-__global__ void __launch_bounds__(kThreads) k_x_inverse_fast(XFast a) {
+// MODE 0: ratio -> forward ; 1: psi update ; 2: plain real output ; 4: the combined update's product.
+// What bounds it is the loads in flight: with the half spectra and the operand rows in registers it had
+// room for two blocks per SM. Gathered by asynchronous copies, the update runs four blocks (256x256x128:
+// 66 -> 32 us), the ratio, which holds its operand row beside the line, three (512x512x64 with 2, 3 and 4
+// blocks 96, 85 and 113 us).
+template <int L, int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == 0 ? 3 : 4) k_x_inverse_fast(const __grid_constant__ XFast a) {
     extern __shared__ float2 sm[];
     fast_x_inverse_tile<L, MODE, false>(a, blockIdx.x, sm);
 }

@@ -8,6 +8,7 @@
 
 #include "dd.cuh"
 #include "fft_fast.cuh"
+#include "lines.cuh"
 
 namespace mvd {
 
@@ -124,42 +125,33 @@ __device__ __forceinline__ void x_store_halves(const XFast& a, float2 (&v)[kE], 
     }
 }
 
-// read both half spectra of each pair and build Z = A + i B (natural order)
+// Read both half spectra of each pair and build Z = A + i B (natural order). They are
+// gathered by asynchronous copies, all in flight at once and in no registers; row r
+// (r < P: A of pair r, else B of pair r - P) sits at the odd stride XH, so that a warp's
+// rows of one k and a line's ascending and descending runs both fall on distinct banks.
 template <int L, bool CO>
 __device__ __forceinline__ void x_load_packed(const XFast& a, float2 (&v)[kE], float2* sm, int p, int t, long rho0,
                                               int nrows) {
-    constexpr int TPL = L / kE, P = kFastThreads / TPL, LS = line_stride(L), XH = L / 2 + 1;
-    constexpr int NTOT = XH * 2 * P, NIT = (NTOT + kFastThreads - 1) / kFastThreads;
-    // rows < P -> line p (A), rows >= P -> line P + p (B); all loads of a
-    // thread are issued before the first shared-memory store
-    float2 tmp[NIT];
-#pragma unroll
-    for (int i = 0; i < NIT; ++i) {
-        const int idx = threadIdx.x + i * kFastThreads;
+    constexpr int TPL = L / kE, P = kFastThreads / TPL, XH = L / 2 + 1;
+    static_assert(2 * P * XH <= P * line_stride(L), "the gathered rows exceed the lines' buffer");
+    const float2* spec = a.spec + rho0;
+    for (int idx = threadIdx.x; idx < XH * 2 * P; idx += kFastThreads) {
         const int k = idx / (2 * P), row = idx - k * 2 * P;
-        tmp[i] = make_float2(0.f, 0.f);
-        if (idx < NTOT && row < nrows) {
-            const long at = (long)k * a.YZ + rho0 + row;
-            tmp[i] = ld2<CO>(a.spec + at);
-        }
+        const bool ok = row < nrows;
+        if constexpr (CO)  // an 8-byte asynchronous copy would go through L1
+            sm[row * XH + k] = ok ? ld2<CO>(spec + (long)k * a.YZ + row) : make_float2(0.f, 0.f);
+        else
+            cp_async8(sm + row * XH + k, ok ? spec + (long)k * a.YZ + row : a.spec, ok);
     }
-#pragma unroll
-    for (int i = 0; i < NIT; ++i) {
-        const int idx = threadIdx.x + i * kFastThreads;
-        const int k = idx / (2 * P), row = idx - k * 2 * P;
-        if (idx < NTOT) sm[row * LS + pad16(k)] = tmp[i];
-    }
+    cp_async_wait_all();
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kE; ++q) {
         const int k = t + TPL * q;
-        if (k <= L / 2) {
-            const float2 A = sm[p * LS + pad16(k)], B = sm[(P + p) * LS + pad16(k)];
-            v[q] = make_float2(A.x - B.y, A.y + B.x);
-        } else {
-            const float2 A = sm[p * LS + pad16(L - k)], B = sm[(P + p) * LS + pad16(L - k)];
-            v[q] = make_float2(A.x + B.y, B.x - A.y);  // conj(A) + i conj(B)
-        }
+        const int kk = k <= L / 2 ? k : L - k;
+        const float2 A = sm[p * XH + kk], B = sm[(P + p) * XH + kk];
+        v[q] = k <= L / 2 ? make_float2(A.x - B.y, A.y + B.x)
+                          : make_float2(A.x + B.y, B.x - A.y);  // conj(A) + i conj(B)
     }
     __syncthreads();
 }
@@ -192,27 +184,21 @@ __device__ __forceinline__ void fast_x_inverse_tile(const XFast& a, long tile, f
     const long rho0 = tile * 2 * P;
     const int nrows = (int)min((long)2 * P, a.YZ - rho0);
     const bool oka = p < nrows, okb = P + p < nrows;
+    // the epilogue's operand rows (phi for the ratio, psi for the update) come into L2
+    // meanwhile: loaded here they would hold 32 registers through the transform
+    if (MODE == 0) prefetch_rows(a.phi + rho0 * L, nrows * L * 4);
+    if (MODE == 1 || MODE == 4) prefetch_rows(a.psi + rho0 * L, nrows * L * 4);
     float2 v[kE];
     x_load_packed<L, CO>(a, v, sm, p, t, rho0, nrows);
     const long ra = (rho0 + p) * L, rb = (rho0 + P + p) * L;
-    // the epilogue's operand rows (phi for the ratio, psi for the update) are
-    // fetched now so that their loads overlap the inverse transform
-    float2 w[kE];
+    LineFFT<L, +1, true>::run(v, sm + p * LS, t, a.tw);
     if (MODE == 0) {
+        float2 w[kE];  // all loads before the first division (whose slow path is a branch)
 #pragma unroll
         for (int q = 0; q < kE; ++q) {
             const int n = t + TPL * q;
             w[q] = make_float2(oka ? __ldg(a.phi + ra + n) : 0.f, okb ? __ldg(a.phi + rb + n) : 0.f);
         }
-    } else if (MODE == 1 || MODE == 4) {
-#pragma unroll
-        for (int q = 0; q < kE; ++q) {
-            const int n = t + TPL * q;
-            w[q] = make_float2(oka ? ld1<CO>(a.psi + ra + n) : 0.f, okb ? ld1<CO>(a.psi + rb + n) : 0.f);
-        }
-    }
-    LineFFT<L, +1, true>::run(v, sm + p * LS, t, a.tw);
-    if (MODE == 0) {
 #pragma unroll
         for (int q = 0; q < kE; ++q) {
             // r - 1 (see the generic ratio pass): the update adds the 1 back
@@ -228,13 +214,14 @@ __device__ __forceinline__ void fast_x_inverse_tile(const XFast& a, long tile, f
             const int n = t + TPL * q;
             if (MODE == 1) {
                 // v = c - 1 (weights and regularisation: update_factor)
-                if (oka)
-                    a.psi[ra + n] = fmaxf(w[q].x * update_factor(v[q].x, w[q].x, a.wt, ra + n, a.lam, a.inv_s), a.eps);
-                if (okb)
-                    a.psi[rb + n] = fmaxf(w[q].y * update_factor(v[q].y, w[q].y, a.wt, rb + n, a.lam, a.inv_s), a.eps);
+                const float pa = oka ? ld1<CO>(a.psi + ra + n) : 0.f, pb = okb ? ld1<CO>(a.psi + rb + n) : 0.f;
+                if (oka) a.psi[ra + n] = fmaxf(pa * update_factor(v[q].x, pa, a.wt, ra + n, a.lam, a.inv_s), a.eps);
+                if (okb) a.psi[rb + n] = fmaxf(pb * update_factor(v[q].y, pb, a.wt, rb + n, a.lam, a.inv_s), a.eps);
             } else if (MODE == 4) {  // combined update: multiply this view's factor into the product
-                if (oka) a.psi[ra + n] = w[q].x * (v[q].x + 1.f) * (a.inv_s ? __ldg(a.inv_s + ra + n) : 1.f);
-                if (okb) a.psi[rb + n] = w[q].y * (v[q].y + 1.f) * (a.inv_s ? __ldg(a.inv_s + rb + n) : 1.f);
+                if (oka)
+                    a.psi[ra + n] = ld1<CO>(a.psi + ra + n) * (v[q].x + 1.f) * (a.inv_s ? __ldg(a.inv_s + ra + n) : 1.f);
+                if (okb)
+                    a.psi[rb + n] = ld1<CO>(a.psi + rb + n) * (v[q].y + 1.f) * (a.inv_s ? __ldg(a.inv_s + rb + n) : 1.f);
             } else {
                 if (oka) a.psi[ra + n] = v[q].x;
                 if (okb) a.psi[rb + n] = v[q].y;
