@@ -295,4 +295,49 @@ struct DftP<9, S> {
     }
 };
 
+// length 16 as 4 x 4: radix 4 over n1 for each n2 (n = 4 n1 + n2), twiddles
+// exp(S 2 pi i n2 k1 / 16), radix 4 over n2 (k = k1 + 4 k2). Inputs bounded by 2^18 q:
+// the first sums reach 2^20.5 q (the products' range is 2^22 q), the outputs 2^22.5 q.
+template <int S>
+struct DftP<16, S> {
+    __device__ __forceinline__ static cdp mul(cdp x, dd r, dd i, f2 c) {  // x (r + i S i)
+        const cdp xs{f2_swap(x.h), f2_swap(x.l)};
+        const float ih = S * i.hi, il = S * i.lo;
+        return cdp_add(cdp_mulk(x, r, c), cdp_mulk(xs, f2_of(-ih, ih), f2_of(-il, il), c));
+    }
+    __device__ __forceinline__ static void run(cdp* v, f2 c) {
+        const dd c1 = MVD_DD(0.92387953251128675613), s1 = MVD_DD(0.38268343236508977173);
+        const dd nc1 = MVD_DD(-0.92387953251128675613), ns1 = MVD_DD(-0.38268343236508977173);
+        const dd h = MVD_DD(0.70710678118654752440), nh = MVD_DD(-0.70710678118654752440);
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+            cdp x[4] = {v[n2], v[n2 + 4], v[n2 + 8], v[n2 + 12]};
+            DftP<4, S>::run(x, c);
+#pragma unroll
+            for (int k1 = 0; k1 < 4; ++k1) v[n2 + 4 * k1] = x[k1];
+        }
+        // v[n2 + 4 k1] times w^(n2 k1)
+        v[5] = mul(v[5], c1, s1, c);
+        v[9] = cdp_mulk(cdp_addi<S>(v[9], v[9]), h, c);
+        v[13] = mul(v[13], s1, c1, c);
+        v[6] = cdp_mulk(cdp_addi<S>(v[6], v[6]), h, c);
+        v[10] = cdp_muli<S>(v[10]);
+        v[14] = cdp_mulk(cdp_addi<-S>(v[14], v[14]), nh, c);
+        v[7] = mul(v[7], s1, c1, c);
+        v[11] = cdp_mulk(cdp_addi<-S>(v[11], v[11]), nh, c);
+        v[15] = mul(v[15], nc1, ns1, c);
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) DftP<4, S>::run(v + 4 * k1, c);
+        // v[4 k1 + k2] -> k1 + 4 k2
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = a + 1; b < 4; ++b) {
+                const cdp t = v[4 * a + b];
+                v[4 * a + b] = v[4 * b + a];
+                v[4 * b + a] = t;
+            }
+    }
+};
+
 }  // namespace mvd

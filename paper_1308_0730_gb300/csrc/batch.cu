@@ -350,8 +350,9 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
             case XR:
             case XU:
                 if (d.fx) {
-                    *ntiles = gen_div_up(d.YZ, 2L * ddf_pairs(d.X));
-                    *elems = 2L * ddf_pairs(d.X) * d.X * 4;
+                    const int pairs = ddf_pairs(d.X, pass == XF ? dd_e(d.X) : kXInvE);
+                    *ntiles = gen_div_up(d.YZ, 2L * pairs);
+                    *elems = 2L * pairs * d.X * 4;
                     return;
                 }
                 *ntiles = dd_x_tiles(d.px, d.YZ);
@@ -633,7 +634,7 @@ mvd_status mvd_batch_create_mode(mvd_ctx* const* ctxs, int n, int n_iter, int mo
         smem = std::max({smem, d.fx ? fast_x_smem(g.X) : gen_smem(gen_x_geo(g.px)), d.fy ? fast_y_smem(g.Y) : gen_smem(gen_line_geo(g.py, 32)),
                          d.fz ? fast_z_smem(g.Z) : gen_smem(gen_line_geo(g.pz, g.Y))});
         if (d.precise)
-            smem = std::max({smem, d.fx ? ddf_ratio_smem(g.X) : dd_smem(dd_x_geo(g.px)), d.fy ? ddf_y_smem(g.Y) : dd_smem(dd_line_geo(g.py, 32)),
+            smem = std::max({smem, d.fx ? std::max(ddf_ratio_smem(g.X), ddf_xf_smem(g.X)) : dd_smem(dd_x_geo(g.px)), d.fy ? ddf_y_smem(g.Y) : dd_smem(dd_line_geo(g.py, 32)),
                              d.fz ? ddf_z_smem(g.Z) : dd_smem(dd_line_geo(g.pz, g.Y))});
     }
     // Entries (default schedule: views 0..nv-1 per iteration). Each volume's

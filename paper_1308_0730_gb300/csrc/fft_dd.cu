@@ -10,7 +10,7 @@ namespace {
 
 // register-resident double-float passes (power-of-two lengths)
 template <int L, int S, int IO = 0>
-__global__ void __launch_bounds__(kDdThreads, 4) k_ddf_y(cdd* S2, long nlines, const cdd* tw2, float2* S1) {
+__global__ void __launch_bounds__(kDdThreads, dd_blocks(dd_e(L))) k_ddf_y(cdd* S2, long nlines, const cdd* tw2, float2* S1) {
     extern __shared__ cdd smd[];
     ddf_y_tile<L, S, false, IO>(S2, nlines, tw2, blockIdx.x, smd, S1);
 }
@@ -23,32 +23,32 @@ __global__ void __launch_bounds__(512) k_ddf_z(cdd* S2, const cdd* K2, int Y, lo
 }
 
 template <int L>
-__global__ void __launch_bounds__(kDdThreads, 2) k_ddf_z2_pipe(cdd* S2, const cdd* K2, int Y, long YZ, int ntiles_y,
+__global__ void __launch_bounds__(z2_threads(L), 3) k_ddf_z2_pipe(cdd* S2, const cdd* K2, int Y, long YZ, int ntiles_y,
                                                               const cdd* tw2, long ntiles) {
     extern __shared__ cdd smd[];
     ddf_z2_pipe<L>(S2, K2, Y, YZ, ntiles_y, tw2, ntiles, smd);
 }
 
 template <int L>
-__global__ void __launch_bounds__(kDdThreads, 4) k_ddf_x_forward(DdXFast a) {
+__global__ void __launch_bounds__(kDdThreads, dd_blocks(dd_e(L))) k_ddf_x_forward(const __grid_constant__ DdXFast a) {
     extern __shared__ cdd smd[];
     ddf_x_forward_tile<L, false>(a, blockIdx.x, smd);
 }
 
 template <int L>
-__global__ void __launch_bounds__(kDdThreads) k_ddf_x_inverse(DdXFast a) {
+__global__ void __launch_bounds__(kDdThreads) k_ddf_x_inverse(const __grid_constant__ DdXFast a) {
     extern __shared__ cdd smd[];
     ddf_x_inverse_tile<L, false>(a, blockIdx.x, smd);
 }
 
 template <int L>
-__global__ void __launch_bounds__(kDdThreads, 4) k_ddf_x_ratio(DdXFast a) {
+__global__ void __launch_bounds__(kDdThreads, dd_blocks(kXInvE)) k_ddf_x_ratio(const __grid_constant__ DdXFast a) {
     extern __shared__ cdd smd[];
     ddf_x_ratio_tile<L, false>(a, blockIdx.x, smd);
 }
 
 template <int L, int MODE>
-__global__ void __launch_bounds__(kDdThreads, 4) k_ddf_x_update(DdXUpd a) {
+__global__ void __launch_bounds__(kDdThreads, dd_blocks(kXInvE)) k_ddf_x_update(const __grid_constant__ DdXUpd a) {
     extern __shared__ cdd smd[];
     ddf_x_update_tile<L, MODE>(a, blockIdx.x, smd);
 }
@@ -114,7 +114,7 @@ mvd_status dd_forward_real(const FftGeom& g, const float* src, cdd* S2, cudaStre
         a.S2 = S2;
         with_dd_len(g.X, [&](auto Lc) {
             constexpr int L = decltype(Lc)::value;
-            rc = launch_raw(k_ddf_x_forward<L>, gen_div_up(g.YZ, 2 * ddf_pairs(L)), kDdThreads, ddf_x_smem(L), st,
+            rc = launch_raw(k_ddf_x_forward<L>, gen_div_up(g.YZ, 2 * ddf_pairs(L, dd_e(L))), kDdThreads, ddf_xf_smem(L), st,
                             "dd x forward (fast)", KC_DD_X_FORWARD, a);
         });
         return rc;
@@ -135,7 +135,7 @@ mvd_status dd_x_inverse_real(const FftGeom& g, const cdd* S2, float* dst, cudaSt
     a.dst = dst;
     with_dd_len(g.X, [&](auto Lc) {
         constexpr int L = decltype(Lc)::value;
-        rc = launch_raw(k_ddf_x_inverse<L>, gen_div_up(g.YZ, 2 * ddf_pairs(L)), kDdThreads, ddf_x_smem(L), st,
+        rc = launch_raw(k_ddf_x_inverse<L>, gen_div_up(g.YZ, 2 * ddf_pairs(L, kXInvE)), kDdThreads, ddf_x_smem(L), st,
                         "dd x inverse (fast)", KC_DD_X_RATIO, a);
     });
     return rc;
@@ -151,7 +151,7 @@ mvd_status dd_x_ratio(const FftGeom& g, cdd* S2, const float* phi, float eps, cu
         a.eps = eps;
         with_dd_len(g.X, [&](auto Lc) {
             constexpr int L = decltype(Lc)::value;
-            rc = launch_raw(k_ddf_x_ratio<L>, gen_div_up(g.YZ, 2 * ddf_pairs(L)), kDdThreads, ddf_ratio_smem(L), st,
+            rc = launch_raw(k_ddf_x_ratio<L>, gen_div_up(g.YZ, 2 * ddf_pairs(L, kXInvE)), kDdThreads, ddf_ratio_smem(L), st,
                             "dd x ratio (fast)", KC_DD_X_RATIO, a);
         });
         return rc;
@@ -192,7 +192,7 @@ mvd_status dd_x_update(const FftGeom& g, const cdd* S2, float* psi, float eps, c
     DdXUpd a{S2, psi, g.YZ, eps, g.tw2x, wt, lam, inv_s};
     with_dd_len(g.X, [&](auto Lc) {
         constexpr int L = decltype(Lc)::value;
-        rc = launch_raw(accumulate ? k_ddf_x_update<L, 4> : k_ddf_x_update<L, 1>, gen_div_up(g.YZ, 2 * ddf_pairs(L)),
+        rc = launch_raw(accumulate ? k_ddf_x_update<L, 4> : k_ddf_x_update<L, 1>, gen_div_up(g.YZ, 2 * ddf_pairs(L, kXInvE)),
                         kDdThreads, ddf_ratio_smem(L), st, "dd x update", KC_X_UPDATE, a);
     });
     return rc;
@@ -203,7 +203,7 @@ static mvd_status ddf_z(const FftGeom& g, cdd* S2, const cdd* K2, dd scale, bool
     with_dd_len(g.Z, [&](auto Lc) {
         constexpr int L = decltype(Lc)::value;
         constexpr int Q = ddf_z_cols(L);
-        const int threads = Q * (L / kE8);
+        const int threads = Q * (L / dd_e(L));
         const int nty = (int)gen_div_up(g.Y, Q);
         rc = launch_raw(mul ? k_ddf_z<L, true> : k_ddf_z<L, false>, (long)g.Xh * nty, threads, ddf_z_smem(L), st,
                         "dd z (fast)", mul ? KC_DD_Z_MUL : KC_SETUP, S2, K2, g.Y, g.YZ, nty, scale, g.tw2z);
@@ -217,12 +217,12 @@ mvd_status dd_z_mul(const FftGeom& g, cdd* S2, const cdd* K2, cudaStream_t st) {
         with_dd_len(g.Z, [&](auto Lc) {
             constexpr int L = decltype(Lc)::value;
             if constexpr (ddf_z2_length(L)) {
-                constexpr int Q = ddf_z_cols(L);
+                constexpr int Q = z2_cols(L);
                 const int nty = (int)gen_div_up(g.Y, Q);
                 const long nt = (long)g.Xh * nty;
                 const size_t smem = ddf_z2_pipe_smem(L);
-                rc = launch_raw(k_ddf_z2_pipe<L>, persistent_grid(k_ddf_z2_pipe<L>, Q * (L / kE8), smem, nt),
-                                Q * (L / kE8), smem, st, "dd z", KC_DD_Z_MUL, S2, K2, g.Y, g.YZ, nty, g.tw2z, nt);
+                rc = launch_raw(k_ddf_z2_pipe<L>, persistent_grid(k_ddf_z2_pipe<L>, z2_threads(L), smem, nt),
+                                z2_threads(L), smem, st, "dd z", KC_DD_Z_MUL, S2, K2, g.Y, g.YZ, nty, g.tw2z, nt);
             }
         });
         return rc;

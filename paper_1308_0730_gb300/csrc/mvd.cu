@@ -357,31 +357,33 @@ mvd_status setup_fft(mvd_ctx* c) {
         // double-float twiddles w^m = exp(-2 pi i m / L): hi = fl32(w), lo =
         // fl32(w - hi), w in FP64. Per axis the table in natural order (m =
         // 0..L-1), then, for the register-resident passes of a power-of-two L,
-        // the same values in the stage order of their radix-8 plan, then in
-        // the stage order of the axis's mixed-radix plan.
+        // the same values in the stage order of their radix-8 plan, then in the
+        // stage order of the axis's mixed-radix plan, then of the radix-16 plan.
         auto twv = [](long m, int L) {
             const double ang = -2.0 * M_PI * (double)m / (double)L;
             const double cr = std::cos(ang), ci = std::sin(ang);
             const float rh = (float)cr, ih = (float)ci;
             return make_float4(rh, ih, (float)(cr - rh), (float)(ci - ih));  // the order of adp.cuh
         };
-        std::vector<float4> tw2(3 * ((size_t)g.X + g.Y + g.Z), make_float4(0.f, 0.f, 0.f, 0.f));
+        std::vector<float4> tw2(4 * ((size_t)g.X + g.Y + g.Z), make_float4(0.f, 0.f, 0.f, 0.f));
         size_t o = 0;
         for (int a = 0; a < 3; ++a) {
             const int L = Ls[a];
             for (int m = 0; m < L; ++m) tw2[o + m] = twv(m, L);
-            if (L >= 32 && L <= 1024 && (L & (L - 1)) == 0)
+            if (L >= 32 && L <= 1024 && (L & (L - 1)) == 0) {
                 stage_ordered_twiddles(L, pow_plan(L, 8), [&](size_t i, long m) { tw2[o + L + i] = twv(m, L); });
+                stage_ordered_twiddles(L, pow_plan(L, 16), [&](size_t i, long m) { tw2[o + 3 * (size_t)L + i] = twv(m, L); });
+            }
             stage_ordered_twiddles(L, plan_radices(*plans[a]),
                                    [&](size_t i, long m) { tw2[o + 2 * (size_t)L + i] = twv(m, L); });
-            o += 3 * (size_t)L;
+            o += 4 * (size_t)L;
         }
         MVD_TRY(dev_alloc(reinterpret_cast<float4**>(&c->d_tw2), tw2.size(), "double-float twiddle tables"));
         MVD_CUDA(cudaMemcpyAsync(c->d_tw2, tw2.data(), tw2.size() * sizeof(float4), cudaMemcpyHostToDevice,
                                  c->stream));
         g.tw2x = c->d_tw2;
-        g.tw2y = reinterpret_cast<const cdd*>(reinterpret_cast<const float4*>(c->d_tw2) + 3 * g.X);
-        g.tw2z = reinterpret_cast<const cdd*>(reinterpret_cast<const float4*>(c->d_tw2) + 3 * (g.X + g.Y));
+        g.tw2y = reinterpret_cast<const cdd*>(reinterpret_cast<const float4*>(c->d_tw2) + 4 * g.X);
+        g.tw2z = reinterpret_cast<const cdd*>(reinterpret_cast<const float4*>(c->d_tw2) + 4 * (g.X + g.Y));
         MVD_TRY(dev_alloc(reinterpret_cast<float4**>(&c->d_S2), ns, "double-float work spectrum"));
         MVD_TRY(dev_alloc(reinterpret_cast<float4**>(&c->d_KP2), ns * 2 * c->nv, "double-float kernel spectra"));
     }
