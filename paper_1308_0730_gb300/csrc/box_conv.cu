@@ -15,6 +15,7 @@ struct BoxJobs {
 template <int NY>
 __global__ void __launch_bounds__(256, 2) k_box_conv(const __grid_constant__ BoxJobs jobs, int splits) {
     extern __shared__ float4 smem4[];
+    pass_wait();
     const BoxJob& b = jobs.j[blockIdx.y];
     const int nz = 8 / splits;
     const int tx = (b.c.ox + kBcTX - 1) / kBcTX, ty = (b.c.oy + 8 * NY - 1) / (8 * NY), tz = (b.c.oz + nz - 1) / nz;
@@ -82,9 +83,10 @@ mvd_status box_convs(std::vector<BoxJob> jobs, cudaStream_t st) {
             tiles = t > tiles ? t : tiles;
         }
         auto kern = ny == 2 ? k_box_conv<2> : k_box_conv<1>;
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_status(e, "box convolutions");
-        kern<<<dim3((unsigned)tiles, (unsigned)n), 256, smem, st>>>(a, s);
+        e = launch_pass(kern, dim3((unsigned)tiles, (unsigned)n), 256, smem, st, a, s);
+        if (e != cudaSuccess) return cuda_status(e, "box convolutions");
         count_launch();
         MVD_TRY(check_launch("box convolutions"));
     }

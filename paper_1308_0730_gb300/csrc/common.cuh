@@ -62,6 +62,30 @@ mvd_status cuda_status(cudaError_t e, const char* what);
         if (_e != cudaSuccess) return ::mvd::cuda_status(_e, #call); \
     } while (0)
 
+// Launch of a pass with programmatic stream serialisation: the grid is launched when the
+// last block of the stream's previous kernel exits, without waiting for that kernel's
+// completion to reach the front end, and its blocks wait (pass_wait) for it before they
+// touch memory. Every kernel launched this way calls pass_wait first. Measured: a
+// calibration step on 128x128x96 (about 900 launches of 6-20 us) 25.8 -> 21.9 ms, ten
+// iterations of 32^3 556 -> 491 us; letting the next grid start with the running one's
+// first instruction instead (its waiting blocks then hold registers and shared memory) 23.5
+// ms and 534 us.
+template <typename... P, typename... A>
+cudaError_t launch_pass(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+__device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
 // FFT plan: one line length L = prod(radix[s]); tw[m] = exp(-2 pi i m / L)
 // (device table, computed in FP64 on the host and rounded to FP32).

@@ -43,6 +43,7 @@ enum { M_RATIO, M_UPDATE, M_CONV, M_ADD, M_ACCUMULATE };
 template <int NY, int KX>
 __global__ void __launch_bounds__(NY == 1 ? 512 : 256, NY == 1 ? 1 : 3) k_direct(const __grid_constant__ DArgs a) {
     extern __shared__ float4 smem4[];
+    pass_wait();
     bc_tile<NY, KX, true, false>(a.c, blockIdx.x, blockIdx.y, blockIdx.z, a.splits, reinterpret_cast<float*>(smem4),
                                  [&](int x, int y, int z, float acc) {
         const long g = (long)x + (long)a.c.ox * (y + (long)a.c.oy * z);
@@ -92,15 +93,16 @@ mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty 
     a.splits = p.s;
     a.mode = mode;
     auto kern = p.ny == 2 ? kernel_for<2>(c.kx) : kernel_for<1>(c.kx);
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return cuda_status(e, name);
     const int nz = p.planes();
     const dim3 grid((c.ox + kBcTX - 1) / kBcTX, (c.oy + 8 * p.ny - 1) / (8 * p.ny), (c.oz + nz - 1) / nz);
     const int cls = mode == M_RATIO ? KC_DIRECT_RATIO
                                     : (mode == M_UPDATE || mode == M_ACCUMULATE) ? KC_DIRECT_UPDATE : KC_DIRECT_CONV;
     prof_begin(cls, st);
-    kern<<<grid, 32 * p.warps, p.smem, st>>>(a);
+    e = launch_pass(kern, grid, 32 * p.warps, p.smem, st, a);
     prof_end(cls, st);
+    if (e != cudaSuccess) return cuda_status(e, name);
     count_launch();
     return check_launch(name);
 }

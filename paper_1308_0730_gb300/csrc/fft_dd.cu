@@ -12,6 +12,7 @@ namespace {
 template <int L, int S, int IO = 0>
 __global__ void __launch_bounds__(kDdThreads, dd_blocks(dd_e(L))) k_ddf_y(cdd* S2, long nlines, const cdd* tw2, float2* S1) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_y_tile<L, S, false, IO>(S2, nlines, tw2, blockIdx.x, smd, S1);
 }
 
@@ -19,6 +20,7 @@ template <int L, bool MUL>
 __global__ void __launch_bounds__(512) k_ddf_z(cdd* S2, const cdd* K2, int Y, long YZ, int ntiles_y, dd scale,
                                                const cdd* tw2) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_z_tile<L, MUL, false>(S2, K2, Y, YZ, ntiles_y, scale, tw2, blockIdx.x, smd);
 }
 
@@ -26,30 +28,35 @@ template <int L>
 __global__ void __launch_bounds__(z2_threads(L), 3) k_ddf_z2_pipe(cdd* S2, const cdd* K2, int Y, long YZ, int ntiles_y,
                                                               const cdd* tw2, long ntiles) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_z2_pipe<L>(S2, K2, Y, YZ, ntiles_y, tw2, ntiles, smd);
 }
 
 template <int L>
 __global__ void __launch_bounds__(kDdThreads, dd_blocks(dd_e(L))) k_ddf_x_forward(const __grid_constant__ DdXFast a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_x_forward_tile<L, false>(a, blockIdx.x, smd);
 }
 
 template <int L>
 __global__ void __launch_bounds__(kDdThreads) k_ddf_x_inverse(const __grid_constant__ DdXFast a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_x_inverse_tile<L, false>(a, blockIdx.x, smd);
 }
 
 template <int L>
 __global__ void __launch_bounds__(kDdThreads, dd_blocks(kXInvE)) k_ddf_x_ratio(const __grid_constant__ DdXFast a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_x_ratio_tile<L, false>(a, blockIdx.x, smd);
 }
 
 template <int L, int MODE>
 __global__ void __launch_bounds__(kDdThreads, dd_blocks(kXInvE)) k_ddf_x_update(const __grid_constant__ DdXUpd a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     ddf_x_update_tile<L, MODE>(a, blockIdx.x, smd);
 }
 
@@ -75,8 +82,9 @@ mvd_status launch_raw(K kern, long grid, int threads, size_t smem, cudaStream_t 
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e, name);
     prof_begin(cls, st);
-    kern<<<(unsigned)grid, threads, smem, st>>>(args...);
+    e = launch_pass(kern, dim3((unsigned)grid), threads, smem, st, args...);
     prof_end(cls, st);
+    if (e != cudaSuccess) return cuda_status(e, name);
     count_launch();
     return check_launch(name);
 }

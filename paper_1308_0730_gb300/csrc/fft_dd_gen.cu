@@ -13,29 +13,34 @@ constexpr int kDdGenBlocks = 4;
 
 __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_forward(const __grid_constant__ DdX a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     dd_x_forward_tile<false>(a, blockIdx.x, smd);
 }
 
 __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_ratio(const __grid_constant__ DdX a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     dd_x_ratio_tile<false>(a, blockIdx.x, smd);
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_update(const __grid_constant__ DdXU u) {
     extern __shared__ cdd smd[];
+    pass_wait();
     dd_x_update_tile<false, MODE>(u, blockIdx.x, smd);
 }
 
 template <int S, bool F32 = false>
 __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_y(const __grid_constant__ DdY a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     dd_y_tile<false, S, F32>(a, blockIdx.x, smd);
 }
 
 template <bool MUL>
 __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_z(const __grid_constant__ DdZ a) {
     extern __shared__ cdd smd[];
+    pass_wait();
     dd_z_tile<false, MUL>(a, blockIdx.x, smd);
 }
 
@@ -45,8 +50,9 @@ mvd_status launch(K kern, const A& a, const LineGeo& g, long grid, cudaStream_t 
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e, name);
     prof_begin(cls, st);
-    kern<<<(unsigned)grid, g.T, smem, st>>>(a);
+    e = launch_pass(kern, dim3((unsigned)grid), g.T, smem, st, a);
     prof_end(cls, st);
+    if (e != cudaSuccess) return cuda_status(e, name);
     count_launch();
     return check_launch(name);
 }

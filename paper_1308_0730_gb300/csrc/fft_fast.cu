@@ -19,6 +19,7 @@ template <int L, int S>
 __global__ void __launch_bounds__(kThreads) k_y_fast(float2* __restrict__ spec, long nlines,
                                                      const float2* __restrict__ tw) {
     extern __shared__ float2 sm[];
+    pass_wait();
     fast_y_tile<L, S, false>(spec, nlines, tw, blockIdx.x, sm);
 }
 
@@ -31,12 +32,14 @@ template <int L, bool MUL>
 __global__ void __launch_bounds__(512) k_z_fast(float2* __restrict__ spec, const float2* __restrict__ K, int Y,
                                                  long YZ, int ntiles_y, float scale, const float2* __restrict__ tw) {
     extern __shared__ float2 sm[];
+    pass_wait();
     fast_z_tile<L, MUL, false>(spec, K, Y, YZ, ntiles_y, scale, tw, blockIdx.x, sm);
 }
 
 template <int L>
 __global__ void __launch_bounds__(kThreads) k_x_forward_fast(XFast a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     fast_x_forward_tile<L, false>(a, blockIdx.x, sm);
 }
 
@@ -48,6 +51,7 @@ __global__ void __launch_bounds__(kThreads) k_x_forward_fast(XFast a) {
 template <int L, int MODE>
 __global__ void __launch_bounds__(kThreads, MODE == 0 ? 3 : 4) k_x_inverse_fast(const __grid_constant__ XFast a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     fast_x_inverse_tile<L, MODE, false>(a, blockIdx.x, sm);
 }
 
@@ -88,8 +92,12 @@ mvd_status fft_y_fast(const FftGeom& g, float2* S, int inverse, cudaStream_t st)
             return;
         }
         prof_begin(KC_Y, st);
-        kern<<<div_up(nlines, LPC), kThreads, smem, st>>>(S, nlines, g.py.tw);
+        e = launch_pass(kern, dim3(div_up(nlines, LPC)), kThreads, smem, st, S, nlines, g.py.tw);
         prof_end(KC_Y, st);
+        if (e != cudaSuccess) {
+            rc = cuda_status(e, "fft y (fast)");
+            return;
+        }
         count_launch();
         rc = check_launch("fft y (fast)");
     });
@@ -114,10 +122,10 @@ static mvd_status z_fast(const FftGeom& g, float2* S, const float2* K, float sca
             }
             const int cls = mul ? KC_Z_MUL : KC_SETUP;
             prof_begin(cls, st);
-            kern<<<g.Xh * ntiles, threads, smem, st>>>(S, K, g.Y, g.YZ, ntiles, scale, g.pz.tw);
+            e = launch_pass(kern, dim3(g.Xh * ntiles), threads, smem, st, S, K, g.Y, g.YZ, ntiles, scale, g.pz.tw);
             prof_end(cls, st);
             count_launch();
-            rc = check_launch("fft z (fast)");
+            rc = e == cudaSuccess ? check_launch("fft z (fast)") : cuda_status(e, "fft z (fast)");
         }
     });
     return rc;
@@ -139,7 +147,7 @@ static mvd_status x_fast(const FftGeom& g, int mode, const float* src, float2* S
     dispatch_len(g.X, [&](auto Lc) {
         constexpr int L = decltype(Lc)::value;
         constexpr int TPL = L / kE, P = kThreads / TPL;
-        const size_t smem = (size_t)2 * P * line_stride(L) * sizeof(float2);
+        const size_t smem = (size_t)P * line_stride(L) * sizeof(float2);  // the P lines; the 2P gathered half rows fit
         const int grid = div_up(g.YZ, 2 * P);
         void (*kern)(XFast) = nullptr;
         int cls = KC_SETUP;
@@ -164,10 +172,10 @@ static mvd_status x_fast(const FftGeom& g, int mode, const float* src, float2* S
             return;
         }
         prof_begin(cls, st);
-        kern<<<grid, kThreads, smem, st>>>(a);
+        e = launch_pass(kern, dim3(grid), kThreads, smem, st, a);
         prof_end(cls, st);
         count_launch();
-        rc = check_launch("fft x (fast)");
+        rc = e == cudaSuccess ? check_launch("fft x (fast)") : cuda_status(e, "fft x (fast)");
     });
     return rc;
 }

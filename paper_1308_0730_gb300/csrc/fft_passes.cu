@@ -31,29 +31,34 @@ constexpr int kGenBlocks = 4;
 
 __global__ void __launch_bounds__(kGenThreads, kGenBlocks) k_x_forward(const __grid_constant__ GenX a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     gen_x_forward_tile<false>(a, blockIdx.x, sm);
 }
 
 __global__ void __launch_bounds__(kGenThreads, kGenBlocks) k_x_ratio(const __grid_constant__ GenX a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     gen_x_ratio_tile<false>(a, blockIdx.x, sm);
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(kGenThreads, kGenBlocks) k_x_inverse(const __grid_constant__ GenX a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     gen_x_inverse_tile<false, MODE>(a, blockIdx.x, sm);
 }
 
 template <int S>
 __global__ void __launch_bounds__(kGenThreads, kGenBlocks) k_y(const __grid_constant__ GenY a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     gen_y_tile<false, S>(a, blockIdx.x, sm);
 }
 
 template <bool MUL>
 __global__ void __launch_bounds__(kGenThreads, kGenBlocks) k_z(const __grid_constant__ GenZ a) {
     extern __shared__ float2 sm[];
+    pass_wait();
     gen_z_tile<false, MUL>(a, blockIdx.x, sm);
 }
 
@@ -63,8 +68,9 @@ mvd_status launch(K kern, const A& a, long grid, cudaStream_t st, const char* na
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e, name);
     prof_begin(cls, st);
-    kern<<<(unsigned)grid, a.g.T, smem, st>>>(a);
+    e = launch_pass(kern, dim3((unsigned)grid), a.g.T, smem, st, a);
     prof_end(cls, st);
+    if (e != cudaSuccess) return cuda_status(e, name);
     count_launch();
     return check_launch(name);
 }
