@@ -40,8 +40,11 @@ enum { M_RATIO, M_UPDATE, M_CONV, M_ADD, M_ACCUMULATE };
 // M_RATIO: out = phi / max(conv, eps); M_UPDATE: out = max(out . conv, eps); M_CONV: out = conv;
 // M_ADD: out += conv; M_ACCUMULATE: out *= conv (the combined update's product). KX: the box's
 // length in x, 0 for those without a kernel of their own.
-template <int NY, int KX>
-__global__ void __launch_bounds__(NY == 1 ? 512 : 256, NY == 1 ? 1 : 3) k_direct(const __grid_constant__ DArgs a) {
+// Blocks of 256 threads have 80 registers, for three of them per SM: with one kernel for both
+// sizes of block the 8-row tiles took 82 to 103, which left two (97x83x61, 9x9x15: 48.4 against
+// 44.7 us a launch); held to 80, blocks of 512 gain nothing (three updates of 32^3: 69 and 73 us).
+template <int NY, int KX, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 1) k_direct(const __grid_constant__ DArgs a) {
     extern __shared__ float4 smem4[];
     pass_wait();
     bc_tile<NY, KX, true, false>(a.c, blockIdx.x, blockIdx.y, blockIdx.z, a.splits, reinterpret_cast<float*>(smem4),
@@ -64,18 +67,18 @@ __global__ void __launch_bounds__(NY == 1 ? 512 : 256, NY == 1 ? 1 : 3) k_direct
     });
 }
 
-template <int NY>
+template <int NY, int THREADS>
 auto kernel_for(int kx) {
     switch (kx) {  // the short rows, whose loop and remainder would cost as much as their taps
-        case 3: return k_direct<NY, 3>;
-        case 5: return k_direct<NY, 5>;
-        case 7: return k_direct<NY, 7>;
-        case 9: return k_direct<NY, 9>;
-        case 11: return k_direct<NY, 11>;
-        case 13: return k_direct<NY, 13>;
-        case 15: return k_direct<NY, 15>;
-        case 17: return k_direct<NY, 17>;
-        default: return k_direct<NY, 0>;
+        case 3: return k_direct<NY, 3, THREADS>;
+        case 5: return k_direct<NY, 5, THREADS>;
+        case 7: return k_direct<NY, 7, THREADS>;
+        case 9: return k_direct<NY, 9, THREADS>;
+        case 11: return k_direct<NY, 11, THREADS>;
+        case 13: return k_direct<NY, 13, THREADS>;
+        case 15: return k_direct<NY, 15, THREADS>;
+        case 17: return k_direct<NY, 17, THREADS>;
+        default: return k_direct<NY, 0, THREADS>;
     }
 }
 
@@ -92,7 +95,7 @@ mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty 
     c.cy = p.cy;
     a.splits = p.s;
     a.mode = mode;
-    auto kern = p.ny == 2 ? kernel_for<2>(c.kx) : kernel_for<1>(c.kx);
+    auto kern = p.ny == 2 ? kernel_for<2, 256>(c.kx) : p.warps == 8 ? kernel_for<1, 256>(c.kx) : kernel_for<1, 512>(c.kx);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return cuda_status(e, name);
     const int nz = p.planes();
