@@ -26,10 +26,10 @@ __device__ __forceinline__ cdp ld_cdp(const cdd* p) {
 
 // geometry: as gen_x_geo, gen_line_geo with 16-byte elements; the ratio's FP32 lines
 // (stride line_stride_for(X, n, 16)) go two to one double-float line
-__host__ __device__ inline LineGeo dd_x_geo(const FftPlan& p) {
+__host__ __device__ inline LineGeo dd_x_geo(const FftPlan& p, int points = kDdTilePoints) {
     LineGeo g{};
     g.L = p.L;
-    g.ln = tile_lines_log2(p, kDdTilePoints, 32, true);
+    g.ln = tile_lines_log2(p, points, 32, points == kDdTilePoints);
     int least = 2 * x_half_stride(p.L);
     const int f = line_stride_for(p.L, g.n(), 16);
     least = least > f ? least : f;
@@ -37,10 +37,10 @@ __host__ __device__ inline LineGeo dd_x_geo(const FftPlan& p) {
     g.T = tile_threads(p, g.ln);
     return g;
 }
-__host__ __device__ inline LineGeo dd_line_geo(const FftPlan& p, int most) {
+__host__ __device__ inline LineGeo dd_line_geo(const FftPlan& p, int most, int points = kDdTilePoints) {
     LineGeo g{};
     g.L = p.L;
-    g.ln = tile_lines_log2(p, kDdTilePoints, most, true);
+    g.ln = tile_lines_log2(p, points, most, points == kDdTilePoints);
     g.ls = line_stride_for(p.L, g.n(), 8);
     g.T = tile_threads(p, g.ln);
     return g;
@@ -60,9 +60,10 @@ struct DdX {
     float2* S;              // ratio: the FP32 spectrum of r - 1 goes here when set, else into S2
 };
 
-__host__ __device__ inline DdX dd_x_args(int X, long YZ, const FftPlan& plan, const cdd* tw2) {
+__host__ __device__ inline DdX dd_x_args(int X, long YZ, const FftPlan& plan, const cdd* tw2,
+                                         int points = kDdTilePoints) {
     DdX a{};
-    a.g = dd_x_geo(plan);
+    a.g = dd_x_geo(plan, points);
     a.X = X;
     a.Xh = X / 2 + 1;
     a.YZ = YZ;
@@ -70,7 +71,9 @@ __host__ __device__ inline DdX dd_x_args(int X, long YZ, const FftPlan& plan, co
     a.tw2 = tw2;
     return a;
 }
-__host__ __device__ inline long dd_x_tiles(const FftPlan& p, long YZ) { return gen_div_up(YZ, 2 * dd_x_geo(p).n()); }
+__host__ __device__ inline long dd_x_tiles(const FftPlan& p, long YZ, int points = kDdTilePoints) {
+    return gen_div_up(YZ, 2 * dd_x_geo(p, points).n());
+}
 
 // pair p = rows (p, n + p): complex line a + i b, exact in double-float
 template <bool CO>
@@ -204,17 +207,18 @@ struct DdY {
     const float2* S1;  // when set, the lines come from this FP32 spectrum (widened exactly)
 };
 
-__host__ __device__ inline DdY dd_y_args(int Xh, int Z, const FftPlan& plan, const cdd* tw2, cdd* S2) {
+__host__ __device__ inline DdY dd_y_args(int Xh, int Z, const FftPlan& plan, const cdd* tw2, cdd* S2,
+                                         int points = kDdTilePoints) {
     DdY a{};
-    a.g = dd_line_geo(plan, 32);
+    a.g = dd_line_geo(plan, 32, points);
     a.nlines = (long)Xh * Z;
     a.plan = plan;
     a.tw2 = tw2;
     a.S2 = S2;
     return a;
 }
-__host__ __device__ inline long dd_y_tiles(const FftPlan& p, int Xh, int Z) {
-    return gen_div_up((long)Xh * Z, dd_line_geo(p, 32).n());
+__host__ __device__ inline long dd_y_tiles(const FftPlan& p, int Xh, int Z, int points = kDdTilePoints) {
+    return gen_div_up((long)Xh * Z, dd_line_geo(p, 32, points).n());
 }
 
 template <bool CO, int S, bool F32 = false>
@@ -253,9 +257,9 @@ struct DdZ {
 };
 
 __host__ __device__ inline DdZ dd_z_args(int Y, long YZ, const FftPlan& plan, const cdd* tw2, cdd* S2, const cdd* K2,
-                                         dd scale) {
+                                         dd scale, int points = kDdTilePoints) {
     DdZ a{};
-    a.g = dd_line_geo(plan, Y);
+    a.g = dd_line_geo(plan, Y, points);
     a.Y = Y;
     a.ntiles_y = (int)gen_div_up(Y, a.g.n());
     a.YZ = YZ;
@@ -266,8 +270,8 @@ __host__ __device__ inline DdZ dd_z_args(int Y, long YZ, const FftPlan& plan, co
     a.scale = scale;
     return a;
 }
-__host__ __device__ inline long dd_z_tiles(const FftPlan& p, int Y, int Xh) {
-    return (long)Xh * gen_div_up(Y, dd_line_geo(p, Y).n());
+__host__ __device__ inline long dd_z_tiles(const FftPlan& p, int Y, int Xh, int points = kDdTilePoints) {
+    return (long)Xh * gen_div_up(Y, dd_line_geo(p, Y, points).n());
 }
 
 // columns: element z of column q at base + z*Y + q, n consecutive q per tile
