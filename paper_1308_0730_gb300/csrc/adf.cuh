@@ -1,4 +1,6 @@
-// Aligned double-float: the arithmetic of the register-resident FFT lines.
+// Aligned double-float: the arithmetic of the double-float FFT lines, in scalar
+// form (also compiled for the host). The passes run the same operations on packed
+// FP32 pairs (adp.cuh), with the same roundings.
 //
 // A value is the unevaluated sum hi + lo of two FP32 numbers, as in dd.cuh,
 // with one more invariant: every hi of a line is an integer multiple of the

@@ -1,7 +1,7 @@
 // Register-resident double-float line FFT and forward-blur tiles for
-// power-of-two lengths 32..1024 (same scheme as fft_fast.cuh, 8 elements per
-// thread: a line of length L is held by TPL = L/8 threads, thread t owning
-// elements t + TPL*q; radix-8 Stockham stages, then one radix 2 or 4 stage;
+// power-of-two lengths 32..1024 (same scheme as fft_fast.cuh, E = 8 or 16 elements
+// per thread: a line of length L is held by TPL = L/E threads, thread t owning
+// elements t + TPL*q; radix-E Stockham stages, then one of the remaining radix;
 // padded shared-memory exchanges between stages).
 #pragma once
 
@@ -75,7 +75,7 @@ __host__ __device__ constexpr int y_line_stride(int L) { return line_padded(L, d
 // Arithmetic: aligned double-float on packed pairs (adf.cuh, adp.cuh). run() first takes the largest
 // component of the line (a reduction over its threads), puts every value on
 // the grid of that bound's quantum, and each later stage moves to a grid 16
-// times coarser (the growth bound of a radix-8 stage); butterfly sums are then
+// (radix 16: 32) times coarser, the growth bound of its stage; butterfly sums are then
 // exact FP32 adds, and only the products (twiddles, sqrt(2)/2) are rounded
 // back onto the grid. The result is an unevaluated pair per component (hi on
 // the last stage's grid, lo the remainder).
@@ -344,7 +344,7 @@ __device__ __forceinline__ void ddf_y_tile(cdd* __restrict__ S2, long nlines, co
 }
 
 // z: forward, times the double-float kernel spectrum, inverse (MUL); or
-// forward times a scale. Needs Q * L/8 threads.
+// forward times a scale. Needs Q * L/dd_e(L) threads.
 template <int L, bool MUL, bool CO>
 __device__ __forceinline__ void ddf_z_tile(cdd* __restrict__ S2, const cdd* __restrict__ K2, int Y, long YZ,
                                            int ntiles_y, dd scale, const cdd* __restrict__ tw2, long tile, cdd* sm) {
