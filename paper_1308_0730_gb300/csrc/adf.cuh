@@ -192,6 +192,10 @@ __host__ __device__ constexpr int adf_gen_shift(int R) {
     return R == 2 ? 2 : (R <= 5 ? 3 : 4);  // ceil(log2(R sqrt 2)) for R = 2..10
 }
 
+// the grid of a mixed-radix line's second stage, from the bound m of the first stage's
+// outputs (which runs in plain double-float): the twiddle products stay below sqrt(2) m
+__host__ __device__ __forceinline__ int adf_second_exp(float m) { return adf_exp_for<18>(1.5f * m); }
+
 // a * k for an FP32-exact constant k, aligned on c's grid; 4 ops
 __host__ __device__ __forceinline__ dd adf_mulf(dd a, float k, float c) {
     const float h = adf_round(ADF_MUL(a.hi, k), c);

@@ -83,8 +83,8 @@ __device__ void dd_x_forward_tile(const DdX& a, long tile, cdd* sm) {
     const long rho0 = tile * 2 * n;
     const int nrows = (int)min((long)2 * n, a.YZ - rho0);
     const float* src = a.src + rho0 * a.X;
-    const cdd* F = line_transform<-1, cdp, true, true, false, CO>(
-        a.g, a.plan, a.tw2 + 2 * a.X, sm, sm + n * ls, 0, w,
+    const cdd* F = line_transform<-1, cdp, true, false, CO>(
+        a.g, a.plan, a.tw2 + 2 * a.X, sm, sm + n * ls, w,
         [&](int p, int i) {
             return cdp_from(p < nrows ? ld1<CO>(src + p * a.X + i) : 0.f,
                             n + p < nrows ? ld1<CO>(src + (n + p) * a.X + i) : 0.f);
@@ -110,8 +110,8 @@ __device__ __forceinline__ cdd* dd_x_inverse_lines(const DdX& a, long rho0, int 
     }
     cp_async_wait_all();
     __syncthreads();
-    return line_transform<+1, cdp, true, false, true, CO>(
-        a.g, a.plan, a.tw2 + 2 * a.X, sm, H, 0, w,
+    return line_transform<+1, cdp, false, true, CO>(
+        a.g, a.plan, a.tw2 + 2 * a.X, sm, H, w,
         [&](int p, int k) {
             const bool up = k <= a.X / 2;
             const int kk = up ? k : a.X - k;
@@ -139,7 +139,8 @@ __device__ void dd_x_update_tile(const DdXU& u, long tile, cdd* sm) {
     const int n = a.g.n();
     const long rho0 = tile * 2 * n;
     const int nrows = (int)min((long)2 * n, a.YZ - rho0);
-    if (MODE != 0) prefetch_rows(u.psi + rho0 * a.X, nrows * a.X * 4);
+    const long base = rho0 * a.X;
+    if (MODE != 0) prefetch_rows(u.psi + base, nrows * a.X * 4);
     dd_x_inverse_lines<CO>(a, rho0, nrows, sm, w, [&](cdd*, int p, int i, cdp v) {
         const float2 z = cdp_round(v);
         const float cv[2] = {z.x, z.y};  // c - 1 of rows p and n + p
@@ -147,7 +148,7 @@ __device__ void dd_x_update_tile(const DdXU& u, long tile, cdd* sm) {
         for (int h = 0; h < 2; ++h) {
             const int row = p + h * n;
             if (row >= nrows) continue;
-            const long at = (rho0 + row) * a.X + i;
+            const long at = base + (row * a.X + i);
             if (MODE == 0) {
                 u.psi[at] = cv[h];
                 continue;
@@ -184,8 +185,8 @@ __device__ void dd_x_ratio_tile(const DdX& a, long tile, cdd* sm) {
     __syncthreads();
     const float2* R = reinterpret_cast<const float2*>(Rd);
     float2* A = reinterpret_cast<float2*>(Rd == sm ? sm + n * a.g.ls : sm);  // two FP32 buffers in the other one
-    const float2* F = line_transform<-1, float2, false, false, false, CO>(
-        gf, a.plan, a.plan.tw + 3 * a.X, A, A + n * gf.ls, 0, nullptr, [&](int p, int i) { return R[p * gf.ls + i]; },
+    const float2* F = line_transform<-1, float2, false, false, CO>(
+        gf, a.plan, a.plan.tw + 3 * a.X, A, A + n * gf.ls, nullptr, [&](int p, int i) { return R[p * gf.ls + i]; },
         [&](float2* buf, int p, int i, float2 v) { buf[p * gf.ls + i] = v; });
     __syncthreads();
     if (a.S) {
@@ -229,8 +230,8 @@ __device__ void dd_y_tile(const DdY& a, long tile, cdd* sm) {
     const int nl = (int)min((long)n, a.nlines - l0);
     cdd* s = a.S2 + l0 * L;
     const float2* s1 = a.S1 + l0 * L;
-    line_transform<S, cdp, true, true, true, CO>(
-        a.g, a.plan, a.tw2 + 2 * L, sm, sm + n * a.g.ls, 0, w,
+    line_transform<S, cdp, true, true, CO>(
+        a.g, a.plan, a.tw2 + 2 * L, sm, sm + n * a.g.ls, w,
         [&](int l, int i) {
             if (l >= nl) return cdp_zero();
             if constexpr (F32) {
@@ -277,7 +278,7 @@ __host__ __device__ inline long dd_z_tiles(const FftPlan& p, int Y, int Xh, int 
 // columns: element z of column q at base + z*Y + q, n consecutive q per tile
 template <bool CO, bool MUL>
 __device__ void dd_z_tile(const DdZ& a, long tile, cdd* sm) {
-    __shared__ unsigned w[16];
+    __shared__ unsigned w[8];
     const int n = a.g.n(), ls = a.g.ls;
     const int kx = (int)(tile / a.ntiles_y);
     const int y0 = (int)(tile - (long)kx * a.ntiles_y) * n;
@@ -287,25 +288,22 @@ __device__ void dd_z_tile(const DdZ& a, long tile, cdd* sm) {
     const cdd* tw = a.tw2 + 2 * a.g.L;
     auto src = [&](int q, int z) { return q < nq ? ld_cdp<CO>(s + (long)z * a.Y + q) : cdp_zero(); };
     if (!MUL) {
-        line_transform<-1, cdp, true, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, 0, w, src, [&](cdd*, int q, int z, cdp v) {
+        line_transform<-1, cdp, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, w, src, [&](cdd*, int q, int z, cdp v) {
             if (q < nq) cdp_store(s + (long)z * a.Y + q, cdp_scale(v, a.scale));
         });
         return;
     }
-    // the last forward stage multiplies by the kernel spectrum and bounds the product,
-    // whose grid the inverse starts on
+    // the last forward stage multiplies by the kernel spectrum
     const cdd* K = a.K2 + base;
     for (int z = threadIdx.x; z < a.g.L; z += blockDim.x) prefetch_l2(K + (long)z * a.Y);
-    float mx = 0.f;
-    cdd* F = line_transform<-1, cdp, true, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, 0, w, src,
+    cdd* F = line_transform<-1, cdp, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, w, src,
                                            [&](cdd* buf, int q, int z, cdp v) {
                                                if (q < nq) v = cdp_mul_pair(v, cdp_load_cg(K + (long)z * a.Y + q));
-                                               mx = cdp_absmax(v, mx);
                                                cdp_store(buf + q * ls + z, v);
                                            });
-    const int e = adf_exp_for<18>(block_bound(mx, w + 8));
-    line_transform<+1, cdp, false, false, false, CO>(
-        a.g, a.plan, tw, F == sm ? sm + n * ls : sm, F, e, nullptr,
+    __syncthreads();
+    line_transform<+1, cdp, false, false, CO>(
+        a.g, a.plan, tw, F == sm ? sm + n * ls : sm, F, w,
         [&](int q, int z) { return cdp_load(F + q * ls + z); },
         [&](cdd*, int q, int z, cdp v) {
             if (q < nq) cdp_store(s + (long)z * a.Y + q, v);

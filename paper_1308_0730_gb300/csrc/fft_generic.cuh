@@ -90,8 +90,8 @@ __device__ void gen_x_forward_tile(const GenX& a, long tile, float2* sm) {
     const long rho0 = tile * 2 * n;
     const int nrows = (int)min((long)2 * n, a.YZ - rho0);
     const float* src = a.src + rho0 * a.X;
-    const float2* F = line_transform<-1, float2, false, true, false, CO>(
-        a.g, a.plan, a.plan.tw + 3 * a.X, sm, sm + n * ls, 0, nullptr,
+    const float2* F = line_transform<-1, float2, true, false, CO>(
+        a.g, a.plan, a.plan.tw + 3 * a.X, sm, sm + n * ls, nullptr,
         [&](int p, int i) {
             return make_float2(p < nrows ? ld1<CO>(src + p * a.X + i) : 0.f,
                                n + p < nrows ? ld1<CO>(src + (n + p) * a.X + i) : 0.f);
@@ -109,8 +109,8 @@ __device__ __forceinline__ float2* gen_x_inverse_lines(const GenX& a, long rho0,
     float2* H = sm + n * a.g.ls;
     gen_gather<CO>(a, H, rho0, nrows);
     __syncthreads();
-    return line_transform<+1, float2, false, false, true, CO>(
-        a.g, a.plan, a.plan.tw + 3 * a.X, sm, H, 0, nullptr,
+    return line_transform<+1, float2, false, true, CO>(
+        a.g, a.plan, a.plan.tw + 3 * a.X, sm, H, nullptr,
         [&](int p, int k) {
             const bool up = k <= a.X / 2;
             const int kk = up ? k : a.X - k;
@@ -135,8 +135,8 @@ __device__ void gen_x_ratio_tile(const GenX& a, long tile, float2* sm) {
         buf[p * ls + i] = make_float2(ra, rb);
     });
     __syncthreads();
-    const float2* F = line_transform<-1, float2, false, false, false, CO>(
-        a.g, a.plan, a.plan.tw + 3 * a.X, R == sm ? sm + n * ls : sm, R, 0, nullptr,
+    const float2* F = line_transform<-1, float2, false, false, CO>(
+        a.g, a.plan, a.plan.tw + 3 * a.X, R == sm ? sm + n * ls : sm, R, nullptr,
         [&](int p, int i) { return R[p * ls + i]; },
         [&](float2* buf, int p, int i, float2 v) { buf[p * ls + i] = v; });
     __syncthreads();
@@ -198,8 +198,8 @@ __device__ void gen_y_tile(const GenY& a, long tile, float2* sm) {
     const long l0 = tile * n;
     const int nl = (int)min((long)n, a.nlines - l0);
     float2* s = a.S + l0 * L;
-    line_transform<S, float2, false, true, true, CO>(
-        a.g, a.plan, a.plan.tw + 3 * L, sm, sm + n * a.g.ls, 0, nullptr,
+    line_transform<S, float2, true, true, CO>(
+        a.g, a.plan, a.plan.tw + 3 * L, sm, sm + n * a.g.ls, nullptr,
         [&](int l, int i) { return l < nl ? ld2<CO>(s + l * L + i) : make_float2(0.f, 0.f); },
         [&](float2*, int l, int i, float2 v) {
             if (l < nl) s[l * L + i] = v;
@@ -246,7 +246,7 @@ __device__ void gen_z_tile(const GenZ& a, long tile, float2* sm) {
     const float2* tw = a.plan.tw + 3 * a.g.L;
     auto src = [&](int q, int z) { return q < nq ? ld2<CO>(s + (long)z * a.Y + q) : make_float2(0.f, 0.f); };
     if (!MUL) {
-        line_transform<-1, float2, false, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, 0, nullptr, src,
+        line_transform<-1, float2, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, nullptr, src,
                                           [&](float2*, int q, int z, float2 v) {
                                               if (q < nq) s[(long)z * a.Y + q] = cscale(v, a.scale);
                                           });
@@ -254,14 +254,14 @@ __device__ void gen_z_tile(const GenZ& a, long tile, float2* sm) {
     }
     const float2* K = a.K + base;
     for (int z = threadIdx.x; z < a.g.L; z += blockDim.x) prefetch_l2(K + (long)z * a.Y);
-    float2* F = line_transform<-1, float2, false, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, 0, nullptr, src,
+    float2* F = line_transform<-1, float2, false, false, CO>(a.g, a.plan, tw, sm, sm + n * ls, nullptr, src,
                                                   [&](float2* buf, int q, int z, float2 v) {
                                                       buf[q * ls + z] =
                                                           q < nq ? cmul(v, __ldg(K + (long)z * a.Y + q)) : v;
                                                   });
     __syncthreads();
-    line_transform<+1, float2, false, false, false, CO>(
-        a.g, a.plan, tw, F == sm ? sm + n * ls : sm, F, 0, nullptr, [&](int q, int z) { return F[q * ls + z]; },
+    line_transform<+1, float2, false, false, CO>(
+        a.g, a.plan, tw, F == sm ? sm + n * ls : sm, F, nullptr, [&](int q, int z) { return F[q * ls + z]; },
         [&](float2*, int q, int z, float2 v) {
             if (q < nq) s[(long)z * a.Y + q] = v;
         });

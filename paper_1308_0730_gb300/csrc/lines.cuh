@@ -11,9 +11,12 @@
 //     half spectra of an x inverse) and the last stage gives its outputs to one
 //     (global memory, the ratio, the update, the kernel product): no pass over the
 //     tile only loads, multiplies or stores;
-//   - double-float stages all run aligned on the tile's grid (adf.cuh), on packed
-//     pairs: the first stage holds its inputs in registers (one butterfly per thread)
-//     while the block reduces their bound;
+//   - double-float runs on packed pairs: the first stage in plain double-float (its
+//     inputs share no grid), the later ones aligned on the tile's grid (adf.cuh), which
+//     the bound of the first stage's outputs gives. Aligning the inputs instead, with the
+//     worst growth of every stage assumed, costs 1.5 bits in the mean and 3 on lines with
+//     spikes (errors against 80-bit transforms, tests/native/line_host_check.cu), and was
+//     no faster (300x180x150, a view update: 584 us; now 583);
 //   - tiles of up to 1700 points (54 KB with both exchange buffers) and blocks of as
 //     many threads as the second stage has butterflies: four or more per SM; operands
 //     that only the last stage reads are prefetched into L2 when the block starts.
@@ -75,8 +78,9 @@ struct LineV<cdp> {
         return cdp_cmul<S>(x, cdp_load_nc(tw), c);
     }
     __device__ __forceinline__ static cdp align(cdp x, f2 c) { return cdp_align(x, c); }
-    template <int R, int S>
-    __device__ __forceinline__ static void dft(cdp* v, f2 c) {
+    __device__ __forceinline__ static float absmax(cdp x, float m) { return cdp_absmax(x, m); }
+    template <int R, int S, typename C>
+    __device__ __forceinline__ static void dft(cdp* v, C c) {
         DftP<R, S>::run(v, c);
     }
 };
@@ -92,21 +96,22 @@ struct LineV<float2> {
         return cmul(x, twiddle<S>(tw, 0));
     }
     __device__ __forceinline__ static float2 align(float2 x, f2) { return x; }
-    template <int R, int S>
-    __device__ __forceinline__ static void dft(float2* v, f2) {
+    __device__ __forceinline__ static float absmax(float2, float m) { return m; }
+    template <int R, int S, typename C>
+    __device__ __forceinline__ static void dft(float2* v, C) {
         Dft<R, S>::run(v);
     }
 };
 
-// the block's largest value of mx (>= 0), through 8 words of shared memory that no
-// other reduction in flight uses; one block barrier
-__device__ __forceinline__ float block_bound(float mx, unsigned* w) {
+// The block's largest value of mx (>= 0), through 8 words of shared memory: written
+// before a block barrier, read after it
+__device__ __forceinline__ void put_bound(float mx, unsigned* w) {
     const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
     if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = m;
-    __syncthreads();
-    unsigned b = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) b = max(b, w[i]);
-    return __uint_as_float(b);
+}
+__device__ __forceinline__ float get_bound(const unsigned* w) {
+    const unsigned lane = threadIdx.x & 31;  // one word a lane: the loop over the words held more registers
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, lane < blockDim.x >> 5 ? w[lane] : 0u));
 }
 
 // Which butterfly of a stage thread t takes: consecutive threads along the n lines, or
@@ -130,52 +135,25 @@ struct Butterfly {
 };
 
 // First stage: elements j + r L/R of a line from src(line, element), outputs to
-// out(line, element, value). Double-float: without BOUND the grid exponent e is given;
-// with it the block takes it from the inputs (w: block_bound's words), which each
-// thread's first butterfly holds in registers meanwhile (lines above 2048 points have
-// more butterflies than threads: those inputs are read twice).
+// out(line, element, value); mx: the largest component of the thread's outputs.
 // ROWS radices whose stride in shared memory would put a quarter-warp on one or two
 // banks (8, 4, 2) keep the other mapping.
-template <int R, int S, typename V, bool BOUND, bool ROWS, typename Src, typename Out>
-__device__ __forceinline__ void line_first(const LineGeo& g, Src&& src, Out&& out, int& e, unsigned* w) {
+template <int R, int S, typename V, bool ROWS, typename Src, typename Out>
+__device__ __forceinline__ void line_first(const LineGeo& g, Src&& src, Out&& out, float& mx) {
     using T = LineV<V>;
     const int nb = g.L / R, total = nb << g.ln;
     const Butterfly<ROWS && (R == 6 || R % 2 == 1)> bf(g, nb);
-    int t = threadIdx.x, line = 0, j = 0;
-    V v[R];
-    if (t < total) {
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+        int line, j;
         bf.at(t, line, j);
+        V v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = src(line, j + r * nb);
-    }
-    f2 c = 0;
-    if constexpr (T::kAligned) {
-        if constexpr (BOUND) {
-            float mx = 0.f;
-            if (t < total) {
+        T::template dft<R, S>(v, Unaligned{});
 #pragma unroll
-                for (int r = 0; r < R; ++r) mx = cdp_absmax(v[r], mx);
-            }
-            for (int i = t + blockDim.x; i < total; i += blockDim.x) {
-                int l2, j2;
-                bf.at(i, l2, j2);
-                for (int r = 0; r < R; ++r) mx = cdp_absmax(src(l2, j2 + r * nb), mx);
-            }
-            e = adf_exp_for<18>(block_bound(mx, w));
-        }
-        c = f2_dup(adf_const_exp2(e));
-    }
-    while (t < total) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = T::align(v[r], c);
-        T::template dft<R, S>(v, c);
-#pragma unroll
-        for (int r = 0; r < R; ++r) out(line, j * R + r, v[r]);
-        t += blockDim.x;
-        if (t < total) {
-            bf.at(t, line, j);
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = src(line, j + r * nb);
+        for (int r = 0; r < R; ++r) {
+            mx = T::absmax(v[r], mx);
+            out(line, j * R + r, v[r]);
         }
     }
 }
@@ -214,32 +192,21 @@ __device__ __noinline__ void line_middle(const LineGeo& g, const typename LineV<
     line_stage<R, S, V, false>(g, from, Ns, tw, c, [&](int line, int i, V v) { LineV<V>::store(to + line * g.ls + i, v); });
 }
 
-// Any stage, shared buffer to shared buffer (Ns = 1: the first, without twiddles)
+// Any stage, shared buffer to shared buffer (Ns = 1: the first, without twiddles or a
+// grid); returns the largest component of the first stage's outputs
 template <int R, int S, typename V>
-__device__ __noinline__ void line_any(const LineGeo& g, const typename LineV<V>::Mem* from,
-                                      typename LineV<V>::Mem* to, int Ns, const typename LineV<V>::Mem* tw, f2 c) {
+__device__ __noinline__ float line_any(const LineGeo& g, const typename LineV<V>::Mem* from,
+                                       typename LineV<V>::Mem* to, int Ns, const typename LineV<V>::Mem* tw, f2 c) {
     using T = LineV<V>;
-    const int nb = g.L / R, total = nb << g.ln;
-    const float inv_ns = 1.0f / (float)Ns;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int line = t & (g.n() - 1), j = t >> g.ln;
-        const int jq = small_div(j, inv_ns), k = j - jq * Ns;
-        V v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = T::load(from + line * g.ls + j + r * nb);
-        if (Ns > 1) {
-            v[0] = T::align(v[0], c);
-#pragma unroll
-            for (int r = 1; r < R; ++r) v[r] = T::template tmul<S>(v[r], tw + (r - 1) * Ns + k, c);
-        } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = T::align(v[r], c);
-        }
-        T::template dft<R, S>(v, c);
-        const int d = jq * Ns * R + k;
-#pragma unroll
-        for (int r = 0; r < R; ++r) T::store(to + line * g.ls + d + r * Ns, v[r]);
+    float mx = 0.f;
+    if (Ns == 1) {
+        line_first<R, S, V, false>(
+            g, [&](int line, int i) { return T::load(from + line * g.ls + i); },
+            [&](int line, int i, V v) { T::store(to + line * g.ls + i, v); }, mx);
+    } else {
+        line_stage<R, S, V, false>(g, from, Ns, tw, c, [&](int line, int i, V v) { T::store(to + line * g.ls + i, v); });
     }
+    return mx;
 }
 
 // CALL(R) for the plan's radices (10 in FP32 plans only)
@@ -268,38 +235,39 @@ __device__ __noinline__ void line_any(const LineGeo& g, const typename LineV<V>:
 // STAGED: every stage goes through shared memory by the functions above, src and last in
 // loops of their own (the persistent batch kernel: with the stages inlined into all of its
 // passes it took eight minutes to compile).
-template <int S, typename V, bool BOUND, bool RIN, bool ROUT, bool STAGED, typename Src, typename Last>
+template <int S, typename V, bool RIN, bool ROUT, bool STAGED, typename Src, typename Last>
 __device__ __forceinline__ typename LineV<V>::Mem* line_transform(const LineGeo& g, const FftPlan& p,
                                                                   const typename LineV<V>::Mem* tw,
                                                                   typename LineV<V>::Mem* A, typename LineV<V>::Mem* B,
-                                                                  int e, unsigned* w, Src&& src, Last&& last) {
+                                                                  unsigned* w, Src&& src, Last&& last) {
     using T = LineV<V>;
     typename T::Mem *from = A, *to = B;
+    float mx = 0.f;
+    int e = 0;
     if constexpr (STAGED) {
         const int total = g.L << g.ln;
         const Butterfly<RIN> in(g, g.L);
         const Butterfly<ROUT> res(g, g.L);
-        float mx = 0.f;
         for (int t = threadIdx.x; t < total; t += blockDim.x) {
             int line, i;
             in.at(t, line, i);
-            const V v = src(line, i);
-            if constexpr (T::kAligned && BOUND) mx = cdp_absmax(v, mx);
-            T::store(A + line * g.ls + i, v);
+            T::store(A + line * g.ls + i, src(line, i));
         }
-        if constexpr (T::kAligned && BOUND) e = adf_exp_for<18>(block_bound(mx, w));
         __syncthreads();
         int Ns = 1;
         for (int s = 0; s < p.nst; ++s) {
             const int R = p.radix[s];
             f2 c = 0;
             if constexpr (T::kAligned) {
-                if (s > 0) e += adf_gen_shift(p.radix[s - 1]);
+                if (s > 0) e = s == 1 ? adf_second_exp(get_bound(w)) : e + adf_gen_shift(p.radix[s - 1]);
                 c = f2_dup(adf_const_exp2(e));
             }
-#define MVD_CALL(RR) line_any<RR, S, V>(g, from, to, Ns, tw, c)
+#define MVD_CALL(RR) mx = line_any<RR, S, V>(g, from, to, Ns, tw, c)
             MVD_RADIX_SWITCH(R, MVD_CALL)
 #undef MVD_CALL
+            if constexpr (T::kAligned) {
+                if (s == 0) put_bound(mx, w);
+            }
             __syncthreads();
             if (s > 0) tw += (R - 1) * Ns;
             Ns *= R;
@@ -316,12 +284,13 @@ __device__ __forceinline__ typename LineV<V>::Mem* line_transform(const LineGeo&
     }
     if (p.nst > 0) {
         auto out = [&](int line, int i, V v) { T::store(A + line * g.ls + i, v); };
-#define MVD_CALL(RR) line_first<RR, S, V, BOUND, RIN>(g, src, out, e, w)
+#define MVD_CALL(RR) line_first<RR, S, V, RIN>(g, src, out, mx)
         MVD_RADIX_SWITCH(p.radix[0], MVD_CALL)
 #undef MVD_CALL
     } else if ((int)threadIdx.x < g.n()) {  // an axis of length 1
         T::store(A + threadIdx.x * g.ls, src((int)threadIdx.x, 0));
     }
+    if constexpr (T::kAligned) put_bound(mx, w);
     __syncthreads();
     if (p.nst <= 1) {  // a line of at most 10 points
         for (int t = threadIdx.x; t < (g.L << g.ln); t += blockDim.x) {
@@ -330,12 +299,13 @@ __device__ __forceinline__ typename LineV<V>::Mem* line_transform(const LineGeo&
         }
         return to;
     }
+    if constexpr (T::kAligned) e = adf_second_exp(get_bound(w));
     int Ns = p.radix[0];
     for (int s = 1; s < p.nst; ++s) {
         const int R = p.radix[s];
         f2 c = 0;
         if constexpr (T::kAligned) {
-            e += adf_gen_shift(p.radix[s - 1]);
+            if (s > 1) e += adf_gen_shift(p.radix[s - 1]);
             c = f2_dup(adf_const_exp2(e));
         }
         if (s + 1 == p.nst) {
@@ -367,9 +337,9 @@ __device__ __forceinline__ void prefetch_rows(const void* p, int bytes) {
 // The two half spectra A, B of the real rows p and n + p from the transformed complex
 // line z = a + i b of pair p: A = (z_k + conj z_-k) / 2, B = (z_k - conj z_-k) / (2 i)
 __device__ __forceinline__ void unpack_pair(cdp zk, cdp zm, cdp& a, cdp& b) {
-    zm = cdp_conj(zm);  // one grid, below 2^23 q: exact sums
-    a = cdp_half(cdp_add(zk, zm));
-    b = cdp_half(cdp_muli<-1>(cdp_sub(zk, zm)));
+    zm = cdp_conj(zm);  // a line of one stage is on no grid
+    a = cdp_half(cdp_two_add(zk, zm));
+    b = cdp_half(cdp_muli<-1>(cdp_two_sub(zk, zm)));
 }
 __device__ __forceinline__ void unpack_pair(float2 zk, float2 zm, float2& a, float2& b) {
     a = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
@@ -377,8 +347,7 @@ __device__ __forceinline__ void unpack_pair(float2 zk, float2 zm, float2& a, flo
 }
 // and back: the full spectrum of a + i b at k (up: k <= L/2) or at L - k
 __device__ __forceinline__ cdp pack_pair(cdp a, cdp b, bool up) {
-    b = cdp_muli<+1>(b);
-    return up ? cdp_two_add(a, b) : cdp_conj(cdp_two_add(a, cdp_neg(b)));
+    return up ? cdp_two_addi<+1>(a, b) : cdp_conj(cdp_two_addi<-1>(a, b));
 }
 __device__ __forceinline__ float2 pack_pair(float2 a, float2 b, bool up) {
     return up ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, b.x - a.y);
