@@ -401,7 +401,7 @@ mvd_status mvd_autotune(mvd_ctx* ctx, const char* cache_path, mvd_tune_result* o
  *            is held fixed. Volume work runs on the direct engine in FP32
  *            (MVD_ERR_UNSUPPORTED for PSF boxes it cannot stage, or more than
  *            32 views). Synchronises the stream. MVD_ERR_STATE without a
- *            forward run.
+ *            forward run, or when a precompute failed after it.
  */
 mvd_status mvd_unrolled_forward(mvd_ctx* ctx, int n_iter);
 mvd_status mvd_unrolled_backward(mvd_ctx* ctx, const float* grad_psi, float* const* grad_views,

@@ -695,6 +695,10 @@ mvd_status mvd_unrolled_backward(mvd_ctx* c, const float* grad_psi, float* const
         set_error("mvd_unrolled_backward: no unrolled forward run to differentiate");
         return MVD_ERR_STATE;
     }
+    if (c->state < 2) {  // a failed precompute has freed what the forward run used
+        set_error("mvd_unrolled_backward: kernels not precomputed");
+        return MVD_ERR_STATE;
+    }
     if (c->nv > kMaxViews) {
         set_error("mvd_unrolled_backward: at most %d views", kMaxViews);
         return MVD_ERR_UNSUPPORTED;
