@@ -320,7 +320,7 @@ mvd_status corr_to_box(const float* a, const float* b, const int dims[3], const 
                   smem);
         return MVD_ERR_UNSUPPORTED;
     }
-    MVD_CUDA(cudaFuncSetAttribute(k_corr_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MVD_CUDA(cudaFuncSetAttribute(k_corr_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCorrMaxSmem));
     prof_begin(KC_KERNEL_GRAD, st);
     k_corr_partial<<<(unsigned)ntiles, kThreads, smem, st>>>(a, b, X, Y, Z, kd[0], kd[1], kd[2], partial);
     const int T = kd[0] * kd[1] * kd[2];

@@ -714,7 +714,7 @@ mvd_status mvd_batch_create_mode(mvd_ctx* const* ctxs, int n, int n_iter, int mo
                             b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return fail(cuda_status(e, "batch tables"));
-    e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(k_batch);
     if (e != cudaSuccess) return fail(cuda_status(e, "batch kernel attributes"));
     int per_sm = 0, sms = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, kGenThreads, smem);

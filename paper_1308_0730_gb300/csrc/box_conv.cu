@@ -83,7 +83,7 @@ mvd_status box_convs(std::vector<BoxJob> jobs, cudaStream_t st) {
             tiles = t > tiles ? t : tiles;
         }
         auto kern = ny == 2 ? k_box_conv<2> : k_box_conv<1>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) return cuda_status(e, "box convolutions");
         e = launch_pass(kern, dim3((unsigned)tiles, (unsigned)n), 256, smem, st, a, s);
         if (e != cudaSuccess) return cuda_status(e, "box convolutions");

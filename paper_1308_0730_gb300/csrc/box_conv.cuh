@@ -34,7 +34,7 @@
 namespace mvd {
 
 constexpr int kBcTX = 32;
-constexpr size_t kBcMaxSmem = 226 * 1024;
+constexpr size_t kBcMaxSmem = 226 * 1024;  // kMaxDynSmem
 
 // one convolution: input box, tap box, output box; `off` is the input index of
 // (output 0, tap 0) per axis; mir reads the taps reversed on every axis

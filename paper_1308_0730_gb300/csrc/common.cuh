@@ -62,6 +62,16 @@ mvd_status cuda_status(cudaError_t e, const char* what);
         if (_e != cudaSuccess) return ::mvd::cuda_status(_e, #call); \
     } while (0)
 
+// Allows a kernel the most dynamic shared memory that any launch asks for (227 KB less 1 KB
+// for static words), whatever this launch takes. The limit belongs to the function, not to
+// the launch: a smaller one set by another thread between this and the launch, or by a later
+// object of smaller size, would refuse it.
+constexpr size_t kMaxDynSmem = 226 * 1024;
+template <typename K>
+cudaError_t allow_smem(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
+}
+
 // Launch of a pass with programmatic stream serialisation: the grid is launched when the
 // last block of the stream's previous kernel exits, without waiting for that kernel's
 // completion to reach the front end, and its blocks wait (pass_wait) for it before they

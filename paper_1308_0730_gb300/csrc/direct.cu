@@ -96,7 +96,7 @@ mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty 
     a.splits = p.s;
     a.mode = mode;
     auto kern = p.ny == 2 ? kernel_for<2, 256>(c.kx) : p.warps == 8 ? kernel_for<1, 256>(c.kx) : kernel_for<1, 512>(c.kx);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return cuda_status(e, name);
     const int nz = p.planes();
     const dim3 grid((c.ox + kBcTX - 1) / kBcTX, (c.oy + 8 * p.ny - 1) / (8 * p.ny), (c.oz + nz - 1) / nz);

@@ -79,7 +79,7 @@ bool with_dd_len(int L, F&& f) {
 template <typename K, typename... Args>
 mvd_status launch_raw(K kern, long grid, int threads, size_t smem, cudaStream_t st, const char* name, int cls,
                       Args... args) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return cuda_status(e, name);
     prof_begin(cls, st);
     e = launch_pass(kern, dim3((unsigned)grid), threads, smem, st, args...);
@@ -95,7 +95,7 @@ long persistent_grid(K kern, int threads, size_t smem, long ntiles) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kern);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_z(const __grid
 template <typename K, typename A>
 mvd_status launch(K kern, const A& a, const LineGeo& g, long grid, cudaStream_t st, const char* name, int cls) {
     const size_t smem = dd_smem(g);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return cuda_status(e, name);
     prof_begin(cls, st);
     e = launch_pass(kern, dim3((unsigned)grid), g.T, smem, st, a);

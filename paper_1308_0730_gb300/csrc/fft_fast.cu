@@ -86,7 +86,7 @@ mvd_status fft_y_fast(const FftGeom& g, float2* S, int inverse, cudaStream_t st)
         constexpr int TPL = L / kE, LPC = kThreads / TPL;
         const size_t smem = (size_t)LPC * line_stride(L) * sizeof(float2);
         auto kern = inverse ? k_y_fast<L, +1> : k_y_fast<L, -1>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) {
             rc = cuda_status(e, "fft y (fast) attr");
             return;
@@ -115,7 +115,7 @@ static mvd_status z_fast(const FftGeom& g, float2* S, const float2* K, float sca
         const size_t smem = (size_t)Q * line_stride(L) * sizeof(float2);
         if constexpr (L <= 1024) {
             auto kern = mul ? k_z_fast<L, true> : k_z_fast<L, false>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = allow_smem(kern);
             if (e != cudaSuccess) {
                 rc = cuda_status(e, "fft z (fast) attr");
                 return;
@@ -166,7 +166,7 @@ static mvd_status x_fast(const FftGeom& g, int mode, const float* src, float2* S
         } else {
             kern = k_x_inverse_fast<L, 2>;
         }
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) {
             rc = cuda_status(e, "fft x (fast) attr");
             return;

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kGenThreads, kGenBlocks) k_z(const __grid_cons
 template <typename K, typename A>
 mvd_status launch(K kern, const A& a, long grid, cudaStream_t st, const char* name, int cls) {
     const size_t smem = gen_smem(a.g);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return cuda_status(e, name);
     prof_begin(cls, st);
     e = launch_pass(kern, dim3((unsigned)grid), a.g.T, smem, st, a);
