@@ -12,7 +12,7 @@ struct BoxJobs {
 };
 
 // two blocks per SM: the compensated sums take four registers per output
-template <int NY>
+template <int NY, int KX>
 __global__ void __launch_bounds__(256, 2) k_box_conv(const __grid_constant__ BoxJobs jobs, int splits) {
     extern __shared__ float4 smem4[];
     pass_wait();
@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(256, 2) k_box_conv(const __grid_constant__ Box
     const int tx = (b.c.ox + kBcTX - 1) / kBcTX, ty = (b.c.oy + 8 * NY - 1) / (8 * NY), tz = (b.c.oz + nz - 1) / nz;
     const int t = blockIdx.x;
     if (t >= tx * ty * tz) return;
-    bc_tile<NY, 0, false, true>(b.c, t % tx, (t / tx) % ty, t / (tx * ty), splits, reinterpret_cast<float*>(smem4),
+    bc_tile<NY, KX, false, true>(b.c, t % tx, (t / tx) % ty, t / (tx * ty), splits, reinterpret_cast<float*>(smem4),
                              [&](int x, int y, int z, float acc) {
         long g = (long)x + (long)b.c.ox * (y + (long)b.c.oy * z);
         if (b.mirror) g = (long)b.c.ox * b.c.oy * b.c.oz - 1 - g;
@@ -44,30 +44,34 @@ mvd_status box_convs(std::vector<BoxJob> jobs, cudaStream_t st) {
             kz = c.kz > kz ? c.kz : kz;
         }
         // one tile height and split for the batch: the cheapest over all its boxes
-        int ny = 0, s = bc_splits(warps, kz);
+        const int s0 = bc_splits(warps, kz);
+        int ny = 0, s = s0;
         BcPlan plan[kBcMaxJobs];
         size_t smem = 0;
-        for (; ny == 0 && s <= 8; s *= 2) {
-            double best = 0.0;
-            for (int t = 2; t >= 1; t /= 2) {
-                double cost = 0.0;
-                size_t sm = 0;
-                BcPlan ps[kBcMaxJobs];
-                bool ok = true;
-                for (int i = 0; i < n && ok; ++i) {
-                    const BoxConv& c = a.j[i].c;
-                    BcPlan p{};
-                    ok = bc_plan_ny(c.ox, c.oy, c.oz, c.kx, c.ky, c.kz, t, s, 8, &p);
-                    cost += p.cost;
-                    sm = p.smem > sm ? p.smem : sm;
-                    ps[i] = p;
-                }
-                if (ok && (ny == 0 || cost < best)) {
-                    best = cost, ny = t, smem = sm;
-                    for (int i = 0; i < n; ++i) plan[i] = ps[i];
-                }
+        double best = 0.0;
+        auto take = [&](int t, bool pieces) {  // the batch in tiles of 8 t rows, if every box fits and it is cheaper
+            double cost = 0.0;
+            size_t sm = 0;
+            BcPlan ps[kBcMaxJobs];
+            for (int i = 0; i < n; ++i) {
+                const BoxConv& c = a.j[i].c;
+                if (!bc_plan_ny(c.ox, c.oy, c.oz, c.kx, c.ky, c.kz, t, s, 8, ps + i, pieces)) return;
+                cost += ps[i].cost;
+                sm = ps[i].smem > sm ? ps[i].smem : sm;
             }
+            if (ny != 0 && cost >= best) return;
+            best = cost, ny = t, smem = sm;
+            for (int i = 0; i < n; ++i) plan[i] = ps[i];
+        };
+        for (; s <= 8; s *= 2) {
+            take(2, false);
+            take(1, false);
             if (ny) break;
+        }
+        const bool pieces = ny == 0;  // a box of which not one row of taps fits
+        if (pieces) {
+            s = s0;
+            take(1, true);
         }
         if (ny == 0) {
             set_error("compound kernels: a PSF box is too large for the tiled convolution");
@@ -79,10 +83,11 @@ mvd_status box_convs(std::vector<BoxJob> jobs, cudaStream_t st) {
             BoxConv& c = a.j[i].c;
             c.ck = plan[i].ck;
             c.cy = plan[i].cy;
+            c.cx = plan[i].cx;
             const long t = (long)((c.ox + 31) / 32) * ((c.oy + 8 * ny - 1) / (8 * ny)) * ((c.oz + nz - 1) / nz);
             tiles = t > tiles ? t : tiles;
         }
-        auto kern = ny == 2 ? k_box_conv<2> : k_box_conv<1>;
+        auto kern = pieces ? k_box_conv<1, -1> : ny == 2 ? k_box_conv<2, 0> : k_box_conv<1, 0>;
         cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) return cuda_status(e, "box convolutions");
         e = launch_pass(kern, dim3((unsigned)tiles, (unsigned)n), 256, smem, st, a, s);

@@ -34,6 +34,7 @@
 namespace mvd {
 
 constexpr int kBcTX = 32;
+constexpr int kBcPiece = 512;  // taps of a row staged at a time where not one whole row fits
 constexpr size_t kBcMaxSmem = 226 * 1024;  // kMaxDynSmem
 
 // one convolution: input box, tap box, output box; `off` is the input index of
@@ -46,7 +47,7 @@ struct BoxConv {
     int ox, oy, oz;
     int offx, offy, offz;
     int mir;
-    int ck, cy;  // tap planes, and tap rows of each, staged at a time
+    int ck, cy, cx;  // tap planes, tap rows of each and taps of a row staged at a time
 };
 
 __host__ __device__ inline int bc_wx(int kx) { return ((kBcTX + kx - 1 + 3) & ~3) | 4; }  // an odd number of float4
@@ -59,7 +60,7 @@ inline size_t bc_smem(int kx, int ky, int ck, int ny, int nz, int warps) {
 }
 
 struct BcPlan {
-    int ny, s, ck, cy, warps;
+    int ny, s, ck, cy, cx, warps;
     size_t smem;
     double cost;  // SM clocks of the whole grid, for comparing plans
     int planes() const { return warps / s; }
@@ -75,10 +76,12 @@ inline int bc_splits(long warps, int kz) {
 // Staged tap planes and estimated cost of blocks of `warps` warps over tiles of 8 ny
 // rows; false where not even one tap row of one plane fits. Three blocks of eight
 // warps per SM where the staging allows it, else two; boxes of which no whole plane
-// fits are staged a few rows at a time.
-inline bool bc_plan_ny(int ox, int oy, int oz, int kx, int ky, int kz, int ny, int s, int warps, BcPlan* p) {
+// fits are staged a few rows at a time, and (pieces) a piece of a row at a time.
+inline bool bc_plan_ny(int ox, int oy, int oz, int kx_all, int ky, int kz, int ny, int s, int warps, BcPlan* p,
+                       bool pieces = false) {
     const int nz = warps / s;
     if (nz < 1) return false;
+    const int kx = pieces && kx_all > kBcPiece ? kBcPiece : kx_all, np = (kx_all + kx - 1) / kx;
     const size_t want[3] = {74 * 1024, 110 * 1024, kBcMaxSmem};
     int ck = 0;
     for (int i = 0; i < 3 && ck == 0; ++i) {
@@ -92,13 +95,13 @@ inline bool bc_plan_ny(int ox, int oy, int oz, int kx, int ky, int kz, int ny, i
     if (ck == 0)
         for (ck = 1; cy > 0 && bc_smem(kx, cy, 1, ny, nz, warps) > kBcMaxSmem;) cy -= cy > 64 ? 16 : 1;
     if (cy <= 0 || (oy + 8 * ny - 1) / (8 * ny) > 65535) return false;
-    *p = BcPlan{ny, s, ck, cy, warps, bc_smem(kx, cy, ck, ny, nz, warps), 0.0};
+    *p = BcPlan{ny, s, ck, cy, kx, warps, bc_smem(kx, cy, ck, ny, nz, warps), 0.0};
     const long blocks = (long)((ox + 31) / 32) * ((oy + 8 * ny - 1) / (8 * ny)) * ((oz + nz - 1) / nz);
     const int most = 24 / warps;
     int res = (int)((227 * 1024) / (p->smem + 1024));
     res = res > most ? most : res;
-    const double nf = kx / 4 + 1, planes = (double)((kz + s - 1) / s);
-    const double chunks = (double)((kz + ck - 1) / ck) * ((ky + cy - 1) / cy);
+    const double nf = kx / 4 + 1, planes = (double)np * ((kz + s - 1) / s);
+    const double chunks = (double)np * ((kz + ck - 1) / ck) * ((ky + cy - 1) / cy);
     // issue slots of a warp: the FMAs and loads of its (row, output) pairs, about 20 more
     // per row; the copies of its share of the tile's rows and of the taps
     const double sums = planes * (ny * ky * (8.0 * kx + nf) + (ky + ny - 1) * (20.0 + nf));
@@ -117,7 +120,8 @@ inline bool bc_plan_ny(int ox, int oy, int oz, int kx, int ky, int kz, int ny, i
 
 // The cheapest of 16- and 8-row tiles (ny_max limits it) for blocks of eight warps,
 // and of 8-row tiles for sixteen, which read the halo of a small volume's few planes
-// half as often; a box so tall that no tile of nz planes fits takes more splits.
+// half as often; a box so tall that no tile of nz planes fits takes more splits, and one so
+// wide that no row of taps fits (from about 6400) is staged in pieces of rows.
 inline bool bc_plan(int ox, int oy, int oz, int kx, int ky, int kz, int ny_max, BcPlan* best) {
     bool any = false;
     for (int s = bc_splits((long)((ox + 31) / 32) * ((oy + 7) / 8) * oz, kz); s <= 8 && !any; s *= 2)
@@ -127,7 +131,8 @@ inline bool bc_plan(int ox, int oy, int oz, int kx, int ky, int kz, int ny_max, 
                 if (bc_plan_ny(ox, oy, oz, kx, ky, kz, ny, s, warps, &p) && (!any || p.cost < best->cost))
                     *best = p, any = true;
             }
-    return any;
+    return any || bc_plan_ny(ox, oy, oz, kx, ky, kz, 1, bc_splits((long)((ox + 31) / 32) * ((oy + 7) / 8) * oz, kz), 8,
+                             best, true);
 }
 
 // A batch of convolutions of small kernels (zero outside their boxes), one
@@ -161,7 +166,7 @@ __device__ __forceinline__ void bc_taps(float (&acc)[8], const float4& t, const 
 // One input row against the tap rows of outputs 0..NY-1 (tp: output 0's tap row;
 // output o's is o rows earlier). KX > 0: the taps of a row are known at compile
 // time, everything unrolls; KX == 0: nf groups of four and rem more (box sizes are
-// odd: one or three).
+// odd: one or three); KX < 0: a piece of a row, rem may be zero.
 template <int NY, int KX>
 __device__ __forceinline__ void bc_row(const float* in, const float* tp, int kxp, int nf, int rem, float (&acc)[NY][8]) {
     auto ld = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
@@ -192,7 +197,7 @@ __device__ __forceinline__ void bc_row(const float* in, const float* tp, int kxp
             b = ld(in + 4 * nf + 8);
 #pragma unroll
             for (int o = 0; o < NY; ++o) bc_taps<3>(acc[o], ld(tp - o * kxp + 4 * nf), a0, a1, b);
-        } else {
+        } else if (KX == 0 || rem == 1) {
 #pragma unroll
             for (int o = 0; o < NY; ++o) bc_taps<1>(acc[o], ld(tp - o * kxp + 4 * nf), a0, a1, b);
         }
@@ -226,15 +231,18 @@ __device__ __forceinline__ void bc_rows(int lo, int hi, const float* in, const f
 // periodic; else zero outside. COMP: every row's sum is formed on its own, the
 // rows of a plane are added, and the planes' sums are added with compensation
 // (Kahan), so the error does not grow with the box; otherwise a plane's taps are
-// one chain and the planes' sums are added plainly (boxes of the direct engine).
+// one chain and the planes' sums are added plainly (boxes of the direct engine). KX < 0:
+// rows of taps are staged in pieces of j.cx (a multiple of four, or the whole row).
 template <int NY, int KX, bool WRAP, bool COMP, typename Epi>
 __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz, int S, float* smem, Epi&& epi) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lx = lane & 3, ly = lane >> 2;
     const int nw = blockDim.x >> 5, nz = nw / S, s = warp & (S - 1), zl = warp / S;
     const int x0 = bx * kBcTX, y0 = by * 8 * NY, z0 = bz * nz;
-    const int wx = bc_wx(j.kx), kxp = bc_kxp(j.kx);
-    const int nf = j.kx >> 2, rem = j.kx & 3;
+    constexpr bool PIECES = KX < 0;
+    const int px = PIECES ? j.cx : j.kx;
+    const int wx = bc_wx(px), kxp = bc_kxp(px);
+    int nf = px >> 2, rem = px & 3;
     float* tile = smem;
     float* taps = smem + (size_t)wx * (8 * NY + j.cy - 1) * (nz + j.ck - 1);
     const float inv_kxp = 1.0f / (float)kxp;
@@ -244,97 +252,104 @@ __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz
         klo = max(0, -(z0 + j.offz) - (nz - 1));
         khi = min(j.kz, j.iz - (z0 + j.offz));
     }
+    int p0 = 0;                            // first tap of the piece
     auto column = [&](int i, bool& okx) {  // input column of tile column i
-        int gx = x0 + j.offx + i;
+        int gx = x0 + j.offx + (PIECES ? p0 : 0) + i;
         okx = gx >= 0 && gx < j.ix;
         if (WRAP) return gx < 0 ? gx + j.ix : (gx >= j.ix ? min(gx - j.ix, j.ix - 1) : gx);
         return okx ? gx : 0;
     };
     bool oka, okb;
-    const int gxa = column(lane, oka), gxb = column(lane + 32, okb);
+    int gxa = column(lane, oka), gxb = column(lane + 32, okb);
     float acc[NY][8], tot[NY][8], cmp[NY][8];
 #pragma unroll
     for (int o = 0; o < NY; ++o)
 #pragma unroll
         for (int i = 0; i < 8; ++i) tot[o][i] = 0.f, cmp[o][i] = 0.f;
     for (int k0 = klo; k0 < khi; k0 += j.ck)
-        for (int q0 = 0; q0 < j.ky; q0 += j.cy) {
-            const int ck = min(j.ck, khi - k0), cy = min(j.cy, j.ky - q0);
-            const int wy = 8 * NY + cy - 1, rows = (nz + ck - 1) * wy;
-            const int iy0 = y0 + j.offy + q0;  // input row of the tile's first
-            const float inv_cy = 1.0f / (float)cy;
-            // each warp copies every nw-th row; a lane's columns (and their wrap) are the same in every row
-            int p = warp / wy, iy = warp - p * wy;
-            for (int r = warp; r < rows; r += nw) {
-                int gz = z0 + j.offz + k0 + p, gy = iy0 + iy;
-                bool ok = true;
-                if (WRAP) {  // one turn covers every input of a valid output; the rest only needs a valid address
-                    gz = gz < 0 ? gz + j.iz : (gz >= j.iz ? min(gz - j.iz, j.iz - 1) : gz);
-                    gy = gy < 0 ? gy + j.iy : (gy >= j.iy ? min(gy - j.iy, j.iy - 1) : gy);
-                } else {
-                    ok = gz >= 0 && gz < j.iz && gy >= 0 && gy < j.iy;
+        for (int q0 = 0; q0 < j.ky; q0 += j.cy)
+            for (p0 = 0; p0 < (PIECES ? j.kx : 1); p0 += PIECES ? j.cx : 1) {
+                const int ck = min(j.ck, khi - k0), cy = min(j.cy, j.ky - q0);
+                const int nx = PIECES ? min(j.cx, j.kx - p0) : j.kx;  // taps of the piece's rows
+                if constexpr (PIECES) {
+                    gxa = column(lane, oka), gxb = column(lane + 32, okb);
+                    nf = nx >> 2, rem = nx & 3;
                 }
-                const float* row = j.in + (ok ? (long)j.ix * (gy + (long)j.iy * gz) : 0L);
-                float* dst = tile + (size_t)r * wx + lane;
-                cp_async4(dst, row + gxa, WRAP || (ok && oka));
-                if (lane + 32 < wx) cp_async4(dst + 32, row + gxb, WRAP || (ok && okb));
-                for (int i = lane + 64; i < wx; i += 32) {
-                    bool okx;
-                    const int gx = column(i, okx);
-                    cp_async4(dst + i - lane, row + gx, WRAP || (ok && okx));
-                }
-                for (iy += nw; iy >= wy; iy -= wy) ++p;
-            }
-            const int nt = ck * cy * kxp;
-            for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-                const int r = small_div(i, inv_kxp), kx = i - r * kxp;
-                const int kz = small_div(r, inv_cy), ky = r - kz * cy;
-                const bool ok = kx < j.kx;
-                long t = kx + (long)j.kx * (q0 + ky + (long)j.ky * (k0 + kz));
-                if (j.mir) t = (long)j.kx * j.ky * j.kz - 1 - t;
-                cp_async4(taps + i, ok ? j.taps + t : j.taps, ok);
-            }
-            asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-            __syncthreads();
-            int ilo = 0, ihi = cy + NY - 1;  // rows of a thread's window that hold input for some lane
-            if (!WRAP) {
-                ilo = max(0, -iy0 - 7 * NY);
-                ihi = min(ihi, j.iy - iy0);
-            }
-            for (int kk = (s - k0) & (S - 1); kk < ck; kk += S) {
-                const float* in = tile + ((size_t)(zl + kk) * wy + ly * NY + ilo) * wx + 8 * lx;
-                const float* tp = taps + ((size_t)kk * cy + ilo) * kxp;
-                float pl[NY][8];
-#pragma unroll
-                for (int o = 0; o < NY; ++o)
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) acc[o][i] = 0.f, pl[o][i] = 0.f;
-                for (int iy = ilo; iy < ihi; ++iy, in += wx, tp += kxp) {
-                    const int lo = max(0, iy - cy + 1), hi = min(NY - 1, iy);
-                    bc_rows<NY, KX>(lo, hi, in, tp, kxp, nf, rem, acc);
-                    if (COMP) {
-#pragma unroll
-                        for (int o = 0; o < NY; ++o)
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) pl[o][i] += acc[o][i], acc[o][i] = 0.f;
+                const int wy = 8 * NY + cy - 1, rows = (nz + ck - 1) * wy;
+                const int iy0 = y0 + j.offy + q0;  // input row of the tile's first
+                const float inv_cy = 1.0f / (float)cy;
+                // each warp copies every nw-th row; a lane's columns (and their wrap) are the same in every row
+                int p = warp / wy, iy = warp - p * wy;
+                for (int r = warp; r < rows; r += nw) {
+                    int gz = z0 + j.offz + k0 + p, gy = iy0 + iy;
+                    bool ok = true;
+                    if (WRAP) {  // one turn covers every input of a valid output; the rest only needs a valid address
+                        gz = gz < 0 ? gz + j.iz : (gz >= j.iz ? min(gz - j.iz, j.iz - 1) : gz);
+                        gy = gy < 0 ? gy + j.iy : (gy >= j.iy ? min(gy - j.iy, j.iy - 1) : gy);
+                    } else {
+                        ok = gz >= 0 && gz < j.iz && gy >= 0 && gy < j.iy;
                     }
+                    const float* row = j.in + (ok ? (long)j.ix * (gy + (long)j.iy * gz) : 0L);
+                    float* dst = tile + (size_t)r * wx + lane;
+                    cp_async4(dst, row + gxa, WRAP || (ok && oka));
+                    if (lane + 32 < wx) cp_async4(dst + 32, row + gxb, WRAP || (ok && okb));
+                    for (int i = lane + 64; i < wx; i += 32) {
+                        bool okx;
+                        const int gx = column(i, okx);
+                        cp_async4(dst + i - lane, row + gx, WRAP || (ok && okx));
+                    }
+                    for (iy += nw; iy >= wy; iy -= wy) ++p;
                 }
+                const int nt = ck * cy * kxp;
+                for (int i = threadIdx.x; i < nt; i += blockDim.x) {
+                    const int r = small_div(i, inv_kxp), kx = i - r * kxp;
+                    const int kz = small_div(r, inv_cy), ky = r - kz * cy;
+                    const bool ok = kx < nx;
+                    long t = (PIECES ? p0 : 0) + kx + (long)j.kx * (q0 + ky + (long)j.ky * (k0 + kz));
+                    if (j.mir) t = (long)j.kx * j.ky * j.kz - 1 - t;
+                    cp_async4(taps + i, ok ? j.taps + t : j.taps, ok);
+                }
+                asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+                __syncthreads();
+                int ilo = 0, ihi = cy + NY - 1;  // rows of a thread's window that hold input for some lane
+                if (!WRAP) {
+                    ilo = max(0, -iy0 - 7 * NY);
+                    ihi = min(ihi, j.iy - iy0);
+                }
+                for (int kk = (s - k0) & (S - 1); kk < ck; kk += S) {
+                    const float* in = tile + ((size_t)(zl + kk) * wy + ly * NY + ilo) * wx + 8 * lx;
+                    const float* tp = taps + ((size_t)kk * cy + ilo) * kxp;
+                    float pl[NY][8];
 #pragma unroll
-                for (int o = 0; o < NY; ++o)
+                    for (int o = 0; o < NY; ++o)
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                        for (int i = 0; i < 8; ++i) acc[o][i] = 0.f, pl[o][i] = 0.f;
+                    for (int iy = ilo; iy < ihi; ++iy, in += wx, tp += kxp) {
+                        const int lo = max(0, iy - cy + 1), hi = min(NY - 1, iy);
+                        bc_rows<NY, KX>(lo, hi, in, tp, kxp, nf, rem, acc);
                         if (COMP) {
-                            const float y = __fsub_rn(pl[o][i], cmp[o][i]);
-                            const float t = __fadd_rn(tot[o][i], y);
-                            cmp[o][i] = __fsub_rn(__fsub_rn(t, tot[o][i]), y);
-                            tot[o][i] = t;
-                        } else {
-                            tot[o][i] += acc[o][i];
+#pragma unroll
+                            for (int o = 0; o < NY; ++o)
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) pl[o][i] += acc[o][i], acc[o][i] = 0.f;
                         }
                     }
+#pragma unroll
+                    for (int o = 0; o < NY; ++o)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            if (COMP) {
+                                const float y = __fsub_rn(pl[o][i], cmp[o][i]);
+                                const float t = __fadd_rn(tot[o][i], y);
+                                cmp[o][i] = __fsub_rn(__fsub_rn(t, tot[o][i]), y);
+                                tot[o][i] = t;
+                            } else {
+                                tot[o][i] += acc[o][i];
+                            }
+                        }
+                }
+                __syncthreads();
             }
-            __syncthreads();
-        }
     if (S == 1) {
         const int z = z0 + zl;
         if (z >= j.oz) return;

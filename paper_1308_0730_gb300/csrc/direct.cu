@@ -39,7 +39,7 @@ enum { M_RATIO, M_UPDATE, M_CONV, M_ADD, M_ACCUMULATE };
 
 // M_RATIO: out = phi / max(conv, eps); M_UPDATE: out = max(out . conv, eps); M_CONV: out = conv;
 // M_ADD: out += conv; M_ACCUMULATE: out *= conv (the combined update's product). KX: the box's
-// length in x, 0 for those without a kernel of their own.
+// length in x, 0 for those without a kernel of their own, -1 for rows staged in pieces.
 // Blocks of 256 threads have 80 registers, for three of them per SM: with one kernel for both
 // sizes of block the 8-row tiles took 82 to 103, which left two (97x83x61, 9x9x15: 48.4 against
 // 44.7 us a launch); held to 80, blocks of 512 gain nothing (three updates of 32^3: 69 and 73 us).
@@ -93,9 +93,13 @@ mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty 
     }
     c.ck = p.ck;
     c.cy = p.cy;
+    c.cx = p.cx;
     a.splits = p.s;
     a.mode = mode;
-    auto kern = p.ny == 2 ? kernel_for<2, 256>(c.kx) : p.warps == 8 ? kernel_for<1, 256>(c.kx) : kernel_for<1, 512>(c.kx);
+    auto kern = p.cx < c.kx     ? k_direct<1, -1, 256>
+                : p.ny == 2     ? kernel_for<2, 256>(c.kx)
+                : p.warps == 8  ? kernel_for<1, 256>(c.kx)
+                                : kernel_for<1, 512>(c.kx);
     cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return cuda_status(e, name);
     const int nz = p.planes();
