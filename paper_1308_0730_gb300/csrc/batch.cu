@@ -101,6 +101,13 @@ __device__ __forceinline__ void with_len(int L, F&& f) {
     }
 }
 
+// two blocks per SM whatever lengths meet in a launch (228 KB, 1 KB of it reserved per block)
+constexpr size_t kBatchMostSmem = 113 * 1024;
+static_assert(ddf_z_smem(64) <= kBatchMostSmem && ddf_z_smem(128) <= kBatchMostSmem && ddf_z_smem(256) <= kBatchMostSmem,
+              "z tiles of the persistent kernel");
+static_assert(ddf_ratio_smem(64) <= kBatchMostSmem && ddf_ratio_smem(128) <= kBatchMostSmem &&
+              ddf_ratio_smem(256) <= kBatchMostSmem, "x tiles of the persistent kernel");
+
 // precise mode, axes of length 64, 128 or 256: register-resident
 // double-float passes (the same tiles as the single-volume engine)
 __device__ __noinline__ bool run_tile_ddf(const VolDesc& d, int pass, int view, long tile, cdd* sm) {

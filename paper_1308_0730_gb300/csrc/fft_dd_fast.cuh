@@ -307,8 +307,16 @@ __host__ __device__ constexpr int z_line_stride8(int L) {
     // odd; with four columns 2 mod 4
     return ddf_z_cols(L) == 4 ? (line_padded(L, dd_e(L)) & ~3) + (line_padded(L, dd_e(L)) % 4 <= 2 ? 2 : 6) : (line_padded(L, dd_e(L)) + 1) | 1;
 }
+// A second exchange buffer (one barrier per exchange) only with 8 points per thread: the 32
+// and 16 columns of 128 and 256 points with 16 would take 140 KB with it, which leaves one
+// block of 8 warps per SM, in the persistent batch kernel for every volume of the launch.
+// Measured with two and one (and with 8 points and two): eight volumes with Z = 128,
+// persistent, 21.4 -> 14.1 ms (13.9), four with Z = 256 14.5 -> 9.8 (9.5); a spectrum of
+// 256x256x128 (kernel set-up) 34.8 -> 27.7 us (30.7); the product pass at 64x64x1024 53.7 ->
+// 39.1 us (54.5).
+__host__ __device__ constexpr int z_buffers(int L) { return dd_e(L) == 16 ? 1 : 2; }
 __host__ __device__ constexpr size_t ddf_z_smem(int L) {
-    return (size_t)2 * ddf_z_cols(L) * z_line_stride8(L) * sizeof(cdd);
+    return (size_t)z_buffers(L) * ddf_z_cols(L) * z_line_stride8(L) * sizeof(cdd);
 }
 
 // IO selects where the lines come from:
@@ -358,8 +366,9 @@ __device__ __forceinline__ void ddf_z_tile(cdd* __restrict__ S2, const cdd* __re
     cdp v[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) v[i] = ok ? ld_cdp<CO>(S2 + base + (long)(t + TPL * i) * Y) : cdp_zero();
-    using FF = LineFFTDD<L, E, -1, false, Q * z_line_stride8(L), Q>;
-    using FI = LineFFTDD<L, E, +1, false, Q * z_line_stride8(L), Q>;
+    constexpr int DB = z_buffers(L) == 2 ? Q * z_line_stride8(L) : 0;
+    using FF = LineFFTDD<L, E, -1, false, DB, Q>;
+    using FI = LineFFTDD<L, E, +1, false, DB, Q>;
     FF::run(v, line_sm, t, tw2);
     if (MUL) {
 #pragma unroll
