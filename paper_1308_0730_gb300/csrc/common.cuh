@@ -270,7 +270,7 @@ struct mvd_ctx {
     float* d_r = nullptr;      // M (direct-path ratio; scratch for kernel placement)
     float* d_psf = nullptr;    // packed normalised PSFs
     float* d_comp = nullptr;   // packed compound kernels
-    float* d_ktmp = nullptr;   // precompute scratch; MVD_EFFICIENT: Q_w = P_w * P_w^* at w * qstride
+    float* d_ktmp = nullptr;   // MVD_EFFICIENT: Q_w = P_w * P_w^* at w * qstride
     long qstride = 0;
     double* d_red = nullptr;   // reduction scratch
     int* d_flag = nullptr;

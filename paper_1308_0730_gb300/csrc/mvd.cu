@@ -977,15 +977,19 @@ mvd_status mvd_precompute_kernels(mvd_ctx* c, int variant) {
     }
     int group = 1;
     const size_t nq = qmax * (size_t)c->nv, nc = compound_scratch(c->nv, c->kd.data(), variant, &group);
-    MVD_TRY(dev_alloc(&c->d_ktmp, nq + nc, "precompute scratch"));
+    MVD_TRY(dev_alloc(&c->d_ktmp, nq, "autocorrelations"));
     c->qstride = (long)qmax;
     if (variant == MVD_EFFICIENT)
         MVD_TRY(autocorr_all(c->nv, c->d_psf, c->koff.data(), c->kd.data(), c->d_ktmp, (long)qmax, c->stream));
     MVD_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), c->stream));
-    MVD_TRY(build_compounds(c->nv, c->d_psf, c->koff.data(), c->kd.data(), variant, c->d_comp, c->d_ktmp, (long)qmax,
-                            c->d_ktmp + nq, group, c->d_flag, c->stream));
+    float* factors = nullptr;  // of the views built at once: given back before the engine takes its buffers
+    if (nc) MVD_TRY(dev_alloc(&factors, nc, "compound factors"));
     int bad = 0;
-    MVD_TRY(read_flag(c, &bad));
+    mvd_status built = build_compounds(c->nv, c->d_psf, c->koff.data(), c->kd.data(), variant, c->d_comp, c->d_ktmp,
+                                       (long)qmax, factors, group, c->d_flag, c->stream);
+    if (built == MVD_OK) built = read_flag(c, &bad);
+    dev_free(factors);
+    MVD_TRY(built);
     if (bad) {
         set_error("mvd_precompute_kernels: a compound kernel sums to zero");
         return MVD_ERR_ARG;
