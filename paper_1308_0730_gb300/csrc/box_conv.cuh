@@ -22,7 +22,10 @@
 // Measured against one output row per thread with scalar loads (GB300, one launch,
 // us): 32^3 outputs, 13x7x7 box 52.9 -> 8.3; 97x83x61, 9x9x15 222 -> 45;
 // 120x110x100, 15x15x41 about 0.46 of the FMA peak (660 us).
-// The order of each output's sum depends on S only, not on NY or CK.
+// The order of each output's sum in the direct engine depends on S only (and, where not one
+// row of taps fits, on the pieces): not on NY, CK, the warps or the rows staged at a time,
+// whose chains run on from one staging to the next. The compensated sums of the kernel
+// algebra add what each staging gives.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -166,7 +169,7 @@ __device__ __forceinline__ void bc_taps(float (&acc)[8], const float4& t, const 
 // One input row against the tap rows of outputs 0..NY-1 (tp: output 0's tap row;
 // output o's is o rows earlier). KX > 0: the taps of a row are known at compile
 // time, everything unrolls; KX == 0: nf groups of four and rem more (box sizes are
-// odd: one or three); KX < 0: a piece of a row, rem may be zero.
+// odd: one or three); KX < 0: nf and rem of a piece of a row, rem may be zero.
 template <int NY, int KX>
 __device__ __forceinline__ void bc_row(const float* in, const float* tp, int kxp, int nf, int rem, float (&acc)[NY][8]) {
     auto ld = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
@@ -231,15 +234,17 @@ __device__ __forceinline__ void bc_rows(int lo, int hi, const float* in, const f
 // periodic; else zero outside. COMP: every row's sum is formed on its own, the
 // rows of a plane are added, and the planes' sums are added with compensation
 // (Kahan), so the error does not grow with the box; otherwise a plane's taps are
-// one chain and the planes' sums are added plainly (boxes of the direct engine). KX < 0:
-// rows of taps are staged in pieces of j.cx (a multiple of four, or the whole row).
+// one chain and the planes' sums are added plainly (boxes of the direct engine), also
+// where its rows are staged cy at a time. KX < 0: planes are staged in rows, and rows in pieces
+// of j.cx (a multiple of four, or the whole row); kernels without COMP and of other KX take
+// whole planes only (the chains would hold registers through the staging).
 template <int NY, int KX, bool WRAP, bool COMP, typename Epi>
 __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz, int S, float* smem, Epi&& epi) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lx = lane & 3, ly = lane >> 2;
     const int nw = blockDim.x >> 5, nz = nw / S, s = warp & (S - 1), zl = warp / S;
     const int x0 = bx * kBcTX, y0 = by * 8 * NY, z0 = bz * nz;
-    constexpr bool PIECES = KX < 0;
+    constexpr bool PIECES = KX < 0, ROWS = PIECES || COMP, CHAIN = PIECES && !COMP;
     const int px = PIECES ? j.cx : j.kx;
     const int wx = bc_wx(px), kxp = bc_kxp(px);
     int nf = px >> 2, rem = px & 3;
@@ -267,9 +272,9 @@ __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz
 #pragma unroll
         for (int i = 0; i < 8; ++i) tot[o][i] = 0.f, cmp[o][i] = 0.f;
     for (int k0 = klo; k0 < khi; k0 += j.ck)
-        for (int q0 = 0; q0 < j.ky; q0 += j.cy)
+        for (int q0 = 0; q0 < (ROWS ? j.ky : 1); q0 += ROWS ? j.cy : 1)
             for (p0 = 0; p0 < (PIECES ? j.kx : 1); p0 += PIECES ? j.cx : 1) {
-                const int ck = min(j.ck, khi - k0), cy = min(j.cy, j.ky - q0);
+                const int ck = min(j.ck, khi - k0), cy = ROWS ? min(j.cy, j.ky - q0) : j.ky;
                 const int nx = PIECES ? min(j.cx, j.kx - p0) : j.kx;  // taps of the piece's rows
                 if constexpr (PIECES) {
                     gxa = column(lane, oka), gxb = column(lane + 32, okb);
@@ -323,7 +328,10 @@ __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz
 #pragma unroll
                     for (int o = 0; o < NY; ++o)
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) acc[o][i] = 0.f, pl[o][i] = 0.f;
+                        for (int i = 0; i < 8; ++i) {
+                            if (!CHAIN || (q0 == 0 && p0 == 0)) acc[o][i] = 0.f;  // CHAIN: ck is 1, one plane at a time
+                            pl[o][i] = 0.f;
+                        }
                     for (int iy = ilo; iy < ihi; ++iy, in += wx, tp += kxp) {
                         const int lo = max(0, iy - cy + 1), hi = min(NY - 1, iy);
                         bc_rows<NY, KX>(lo, hi, in, tp, kxp, nf, rem, acc);
@@ -343,7 +351,7 @@ __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz
                                 const float t = __fadd_rn(tot[o][i], y);
                                 cmp[o][i] = __fsub_rn(__fsub_rn(t, tot[o][i]), y);
                                 tot[o][i] = t;
-                            } else {
+                            } else if (!CHAIN || (q0 + cy == j.ky && p0 + nx == j.kx)) {
                                 tot[o][i] += acc[o][i];
                             }
                         }

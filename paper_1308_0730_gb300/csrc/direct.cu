@@ -39,7 +39,7 @@ enum { M_RATIO, M_UPDATE, M_CONV, M_ADD, M_ACCUMULATE };
 
 // M_RATIO: out = phi / max(conv, eps); M_UPDATE: out = max(out . conv, eps); M_CONV: out = conv;
 // M_ADD: out += conv; M_ACCUMULATE: out *= conv (the combined update's product). KX: the box's
-// length in x, 0 for those without a kernel of their own, -1 for rows staged in pieces.
+// length in x, 0 for those without a kernel of their own, -1 for planes staged in rows.
 // Blocks of 256 threads have 80 registers, for three of them per SM: with one kernel for both
 // sizes of block the 8-row tiles took 82 to 103, which left two (97x83x61, 9x9x15: 48.4 against
 // 44.7 us a launch); held to 80, blocks of 512 gain nothing (three updates of 32^3: 69 and 73 us).
@@ -78,6 +78,7 @@ auto kernel_for(int kx) {
         case 13: return k_direct<NY, 13, THREADS>;
         case 15: return k_direct<NY, 15, THREADS>;
         case 17: return k_direct<NY, 17, THREADS>;
+        case -1: return k_direct<NY, -1, THREADS>;
         default: return k_direct<NY, 0, THREADS>;
     }
 }
@@ -96,10 +97,8 @@ mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty 
     c.cx = p.cx;
     a.splits = p.s;
     a.mode = mode;
-    auto kern = p.cx < c.kx     ? k_direct<1, -1, 256>
-                : p.ny == 2     ? kernel_for<2, 256>(c.kx)
-                : p.warps == 8  ? kernel_for<1, 256>(c.kx)
-                                : kernel_for<1, 512>(c.kx);
+    const int kx = p.cy < c.ky || p.cx < c.kx ? -1 : c.kx;
+    auto kern = p.ny == 2 ? kernel_for<2, 256>(kx) : p.warps == 8 ? kernel_for<1, 256>(kx) : kernel_for<1, 512>(kx);
     cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return cuda_status(e, name);
     const int nz = p.planes();

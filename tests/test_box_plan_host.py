@@ -64,3 +64,23 @@ def test_every_accepted_box_has_a_tile(plan):
         assert p["cx"] == box[0] or (p["cx"] < box[0] and p["cx"] % 4 == 0), what
         nz = p["warps"] // p["s"]
         assert nz >= 1 and -(-dims[2] // nz) <= 65535 and -(-dims[1] // (8 * p["ny"])) <= 65535, what
+
+
+def test_tile_choice_does_not_change_the_order_of_sums(plan):
+    """Splits of the tap planes and pieces of their rows: the same for ty = 8 and ty = 4. (The rows
+    staged at a time may differ: their chains run on, tests/test_gpu_direct_heights.py.)"""
+    rng = random.Random(5)
+    cases = [((200, 80, 40), (101, 41, 3)), ((194, 356, 87), (1, 191, 3)), ((40, 194, 78), (11, 95, 1))]
+    while len(cases) < 4000:
+        box = tuple(2 * rng.randrange(0, int(10 ** rng.uniform(0.3, 2.0))) + 1 for _ in range(3))
+        if accepted(*box):
+            cases.append((tuple(k + rng.randrange(0, 200) for k in box), box))
+    plans = plan([(dims, box, ty) for dims, box in cases for ty in (8, 4)])
+    heights = rows = 0
+    for (dims, box), a, b in zip(cases, plans[::2], plans[1::2]):
+        assert (a["s"], a["cx"]) == (b["s"], b["cx"]), f"{box} taps on {dims}: {a} and {b}"
+        # a chain runs on over the stagings of one plane only
+        assert all(p["ck"] == 1 or (p["cy"], p["cx"]) == (box[1], box[0]) for p in (a, b)), f"{box} taps on {dims}: {a}, {b}"
+        heights += a["ny"] != b["ny"]
+        rows += a["cy"] != b["cy"]
+    assert heights > 400 and rows > 4  # the two choices do differ in their tiles
