@@ -7,6 +7,8 @@ import subprocess
 
 import pytest
 
+from tests._direct_shapes import TALL_TILES
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_1308_0730_gb300", "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
@@ -84,3 +86,12 @@ def test_tile_choice_does_not_change_the_order_of_sums(plan):
         heights += a["ny"] != b["ny"]
         rows += a["cy"] != b["cy"]
     assert heights > 400 and rows > 4  # the two choices do differ in their tiles
+
+
+def test_shapes_of_the_tall_tiles(plan):
+    """The volumes that test_gpu_direct_tall.py runs do take 16-row tiles."""
+    plans = plan([(dims, box, 8) for dims, box in TALL_TILES])
+    assert all(p["ny"] == 2 for p in plans), plans
+    assert {b[0] for _, b in TALL_TILES} >= {3, 5, 7, 9, 11, 13, 15, 17, 19, 21}
+    assert {p["s"] for p in plans} >= {1, 4, 8}
+    assert plans[-1]["cy"] < TALL_TILES[-1][1][1]
