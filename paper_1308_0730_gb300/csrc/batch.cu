@@ -90,7 +90,7 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
 // persistent kernel runs two blocks of 128 registers per SM (three, at 80, spill: 1537 ms for
 // the 48 volumes), so its tiles are larger than those of the passes' own kernels, which run
 // four: 48 volumes 1246 -> 1028 ms.
-constexpr int kBatchTilePoints = 3200;
+__host__ __device__ constexpr TileRule batch_tile_rule() { return {3200, false}; }
 
 template <typename F>
 __device__ __forceinline__ void with_len(int L, F&& f) {
@@ -178,7 +178,7 @@ __device__ __noinline__ void run_tile_dd(const VolDesc& d, int pass, int view, l
     if (run_tile_ddf(d, pass, view, tile, sm)) return;
     switch (pass) {
         case XF: {
-            DdX a = dd_x_args(d.X, d.YZ, d.px, d.tw2x, kBatchTilePoints);
+            DdX a = dd_x_args(d.X, d.YZ, d.px, d.tw2x, batch_tile_rule());
             a.src = d.psi;
             a.S2 = d.S2;
             t_dd_xf(a, tile, sm);
@@ -186,21 +186,21 @@ __device__ __noinline__ void run_tile_dd(const VolDesc& d, int pass, int view, l
         }
         case YF1:
         case YF2:
-            t_dd_yf(dd_y_args(d.Xh, d.Z, d.py, d.tw2y, d.S2, kBatchTilePoints), tile, sm);
+            t_dd_yf(dd_y_args(d.Xh, d.Z, d.py, d.tw2y, d.S2, batch_tile_rule()), tile, sm);
             break;
         case YI1:
         case YI2:
-            t_dd_yi(dd_y_args(d.Xh, d.Z, d.py, d.tw2y, d.S2, kBatchTilePoints), tile, sm);
+            t_dd_yi(dd_y_args(d.Xh, d.Z, d.py, d.tw2y, d.S2, batch_tile_rule()), tile, sm);
             break;
         case Z1:
         case Z2: {
             const cdd* K2 = reinterpret_cast<const cdd*>(reinterpret_cast<const float4*>(d.KP2) +
                                                          ns * (2 * view + (pass == Z2 ? 1 : 0)));
-            t_dd_z(dd_z_args(d.Y, d.YZ, d.pz, d.tw2z, d.S2, K2, dd{1.f, 0.f}, kBatchTilePoints), tile, sm);
+            t_dd_z(dd_z_args(d.Y, d.YZ, d.pz, d.tw2z, d.S2, K2, dd{1.f, 0.f}, batch_tile_rule()), tile, sm);
             break;
         }
         default: {  // XR
-            DdX a = dd_x_args(d.X, d.YZ, d.px, d.tw2x, kBatchTilePoints);
+            DdX a = dd_x_args(d.X, d.YZ, d.px, d.tw2x, batch_tile_rule());
             a.S2 = d.S2;
             a.phi = d.views + (size_t)view * d.M;
             a.eps = d.eps;
@@ -286,7 +286,7 @@ __device__ __noinline__ void run_tile(const VolDesc& d, int pass, int view, long
                     });
                 } else {
                     DdXU u{};
-                    u.x = dd_x_args(d.X, d.YZ, d.px, d.tw2x, kBatchTilePoints);
+                    u.x = dd_x_args(d.X, d.YZ, d.px, d.tw2x, batch_tile_rule());
                     u.x.S2 = d.S2;
                     u.x.eps = d.eps;
                     u.psi = d.psi;
@@ -368,8 +368,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                     *elems = 2L * pairs * d.X * 4;
                     return;
                 }
-                *ntiles = dd_x_tiles(d.px, d.YZ, kBatchTilePoints);
-                *elems = 2L * dd_x_geo(d.px, kBatchTilePoints).n() * d.X * 4;  // double-float work counts about 4x
+                *ntiles = dd_x_tiles(d.px, d.YZ, batch_tile_rule());
+                *elems = 2L * dd_x_geo(d.px, batch_tile_rule()).n() * d.X * 4;  // double-float work counts about 4x
                 return;
             case Z1:
             case Z2:
@@ -378,8 +378,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                     *elems = (long)ddf_z_cols(d.Z) * d.Z * 4;
                     return;
                 }
-                *ntiles = dd_z_tiles(d.pz, d.Y, d.Xh, kBatchTilePoints);
-                *elems = (long)dd_line_geo(d.pz, d.Y, kBatchTilePoints).n() * d.Z * 4;
+                *ntiles = dd_z_tiles(d.pz, d.Y, d.Xh, batch_tile_rule());
+                *elems = (long)dd_line_geo(d.pz, d.Y, batch_tile_rule()).n() * d.Z * 4;
                 return;
             default:
                 if (d.fy) {
@@ -387,8 +387,8 @@ void pass_tiles(const VolDesc& d, int pass, long* ntiles, long* elems) {
                     *elems = (long)ddf_y_lines(d.Y) * d.Y * 4;
                     return;
                 }
-                *ntiles = dd_y_tiles(d.py, d.Xh, d.Z, kBatchTilePoints);
-                *elems = (long)dd_line_geo(d.py, 32, kBatchTilePoints).n() * d.Y * 4;
+                *ntiles = dd_y_tiles(d.py, d.Xh, d.Z, batch_tile_rule());
+                *elems = (long)dd_line_geo(d.py, 32, batch_tile_rule()).n() * d.Y * 4;
                 return;
         }
     }
@@ -647,8 +647,8 @@ mvd_status mvd_batch_create_mode(mvd_ctx* const* ctxs, int n, int n_iter, int mo
         smem = std::max({smem, d.fx ? fast_x_smem(g.X) : gen_smem(gen_x_geo(g.px)), d.fy ? fast_y_smem(g.Y) : gen_smem(gen_line_geo(g.py, 32)),
                          d.fz ? fast_z_smem(g.Z) : gen_smem(gen_line_geo(g.pz, g.Y))});
         if (d.precise)
-            smem = std::max({smem, d.fx ? std::max(ddf_ratio_smem(g.X), ddf_xf_smem(g.X)) : dd_smem(dd_x_geo(g.px, kBatchTilePoints)), d.fy ? ddf_y_smem(g.Y) : dd_smem(dd_line_geo(g.py, 32, kBatchTilePoints)),
-                             d.fz ? ddf_z_smem(g.Z) : dd_smem(dd_line_geo(g.pz, g.Y, kBatchTilePoints))});
+            smem = std::max({smem, d.fx ? std::max(ddf_ratio_smem(g.X), ddf_xf_smem(g.X)) : dd_smem(dd_x_geo(g.px, batch_tile_rule())), d.fy ? ddf_y_smem(g.Y) : dd_smem(dd_line_geo(g.py, 32, batch_tile_rule())),
+                             d.fz ? ddf_z_smem(g.Z) : dd_smem(dd_line_geo(g.pz, g.Y, batch_tile_rule()))});
     }
     // Entries (default schedule: views 0..nv-1 per iteration). Each volume's
     // own entries stay in order; across volumes they are merged by the

@@ -26,10 +26,10 @@ __device__ __forceinline__ cdp ld_cdp(const cdd* p) {
 
 // geometry: as gen_x_geo, gen_line_geo with 16-byte elements; the ratio's FP32 lines
 // (stride line_stride_for(X, n, 16)) go two to one double-float line
-__host__ __device__ inline LineGeo dd_x_geo(const FftPlan& p, int points = kDdTilePoints) {
+__host__ __device__ inline LineGeo dd_x_geo(const FftPlan& p, TileRule rule = dd_tile_rule()) {
     LineGeo g{};
     g.L = p.L;
-    g.ln = tile_lines_log2(p, points, 32, points == kDdTilePoints);
+    g.ln = tile_lines_log2(p, rule, 32);
     int least = 2 * x_half_stride(p.L);
     const int f = line_stride_for(p.L, g.n(), 16);
     least = least > f ? least : f;
@@ -37,10 +37,10 @@ __host__ __device__ inline LineGeo dd_x_geo(const FftPlan& p, int points = kDdTi
     g.T = tile_threads(p, g.ln);
     return g;
 }
-__host__ __device__ inline LineGeo dd_line_geo(const FftPlan& p, int most, int points = kDdTilePoints) {
+__host__ __device__ inline LineGeo dd_line_geo(const FftPlan& p, int most, TileRule rule = dd_tile_rule()) {
     LineGeo g{};
     g.L = p.L;
-    g.ln = tile_lines_log2(p, points, most, points == kDdTilePoints);
+    g.ln = tile_lines_log2(p, rule, most);
     g.ls = line_stride_for(p.L, g.n(), 8);
     g.T = tile_threads(p, g.ln);
     return g;
@@ -61,9 +61,9 @@ struct DdX {
 };
 
 __host__ __device__ inline DdX dd_x_args(int X, long YZ, const FftPlan& plan, const cdd* tw2,
-                                         int points = kDdTilePoints) {
+                                         TileRule rule = dd_tile_rule()) {
     DdX a{};
-    a.g = dd_x_geo(plan, points);
+    a.g = dd_x_geo(plan, rule);
     a.X = X;
     a.Xh = X / 2 + 1;
     a.YZ = YZ;
@@ -71,8 +71,8 @@ __host__ __device__ inline DdX dd_x_args(int X, long YZ, const FftPlan& plan, co
     a.tw2 = tw2;
     return a;
 }
-__host__ __device__ inline long dd_x_tiles(const FftPlan& p, long YZ, int points = kDdTilePoints) {
-    return gen_div_up(YZ, 2 * dd_x_geo(p, points).n());
+__host__ __device__ inline long dd_x_tiles(const FftPlan& p, long YZ, TileRule rule = dd_tile_rule()) {
+    return gen_div_up(YZ, 2 * dd_x_geo(p, rule).n());
 }
 
 // pair p = rows (p, n + p): complex line a + i b, exact in double-float
@@ -209,17 +209,17 @@ struct DdY {
 };
 
 __host__ __device__ inline DdY dd_y_args(int Xh, int Z, const FftPlan& plan, const cdd* tw2, cdd* S2,
-                                         int points = kDdTilePoints) {
+                                         TileRule rule = dd_tile_rule()) {
     DdY a{};
-    a.g = dd_line_geo(plan, 32, points);
+    a.g = dd_line_geo(plan, 32, rule);
     a.nlines = (long)Xh * Z;
     a.plan = plan;
     a.tw2 = tw2;
     a.S2 = S2;
     return a;
 }
-__host__ __device__ inline long dd_y_tiles(const FftPlan& p, int Xh, int Z, int points = kDdTilePoints) {
-    return gen_div_up((long)Xh * Z, dd_line_geo(p, 32, points).n());
+__host__ __device__ inline long dd_y_tiles(const FftPlan& p, int Xh, int Z, TileRule rule = dd_tile_rule()) {
+    return gen_div_up((long)Xh * Z, dd_line_geo(p, 32, rule).n());
 }
 
 template <bool CO, int S, bool F32 = false>
@@ -258,9 +258,9 @@ struct DdZ {
 };
 
 __host__ __device__ inline DdZ dd_z_args(int Y, long YZ, const FftPlan& plan, const cdd* tw2, cdd* S2, const cdd* K2,
-                                         dd scale, int points = kDdTilePoints) {
+                                         dd scale, TileRule rule = dd_tile_rule()) {
     DdZ a{};
-    a.g = dd_line_geo(plan, Y, points);
+    a.g = dd_line_geo(plan, Y, rule);
     a.Y = Y;
     a.ntiles_y = (int)gen_div_up(Y, a.g.n());
     a.YZ = YZ;
@@ -271,8 +271,8 @@ __host__ __device__ inline DdZ dd_z_args(int Y, long YZ, const FftPlan& plan, co
     a.scale = scale;
     return a;
 }
-__host__ __device__ inline long dd_z_tiles(const FftPlan& p, int Y, int Xh, int points = kDdTilePoints) {
-    return (long)Xh * gen_div_up(Y, dd_line_geo(p, Y, points).n());
+__host__ __device__ inline long dd_z_tiles(const FftPlan& p, int Y, int Xh, TileRule rule = dd_tile_rule()) {
+    return (long)Xh * gen_div_up(Y, dd_line_geo(p, Y, rule).n());
 }
 
 // columns: element z of column q at base + z*Y + q, n consecutive q per tile

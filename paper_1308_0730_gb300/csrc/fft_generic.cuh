@@ -25,7 +25,7 @@ __host__ __device__ inline int x_half_stride(int X) { return (X / 2 + 1) | 1; }
 __host__ __device__ inline LineGeo gen_x_geo(const FftPlan& p) {
     LineGeo g{};
     g.L = p.L;
-    g.ln = tile_lines_log2(p, kF32TilePoints, 32, false);
+    g.ln = tile_lines_log2(p, f32_tile_rule(), 32);
     const int hs = 2 * x_half_stride(p.L);  // 2n staged rows share one exchange buffer
     g.ls = line_stride_for(p.L > hs ? p.L : hs, g.n(), 16);
     g.T = tile_threads(p, g.ln);
@@ -34,7 +34,7 @@ __host__ __device__ inline LineGeo gen_x_geo(const FftPlan& p) {
 __host__ __device__ inline LineGeo gen_line_geo(const FftPlan& p, int most) {
     LineGeo g{};
     g.L = p.L;
-    g.ln = tile_lines_log2(p, kF32TilePoints, most, false);
+    g.ln = tile_lines_log2(p, f32_tile_rule(), most);
     g.ls = line_stride_for(p.L, g.n(), 16);
     g.T = tile_threads(p, g.ln);
     return g;

@@ -47,12 +47,23 @@ struct LineGeo {
     __host__ __device__ int n() const { return 1 << ln; }
 };
 
-// lines per tile: the largest power of two whose points fit `points` and, for
-// double-float, whose first-stage butterflies fit 256 threads (at most `most` lines)
-__host__ __device__ inline int tile_lines_log2(const FftPlan& p, int points, int most, bool dd) {
+// What a pass's tiles may hold: points, and whether a tile's first-stage butterflies are at
+// most 256, one for each thread of a block (a second, mostly empty round of them took
+// 100x108x72 from 120 to 127 us a view update)
+struct TileRule {
+    int points;
+    bool one_round;
+};
+__host__ __device__ constexpr TileRule dd_tile_rule() { return {1700, true}; }
+__host__ __device__ constexpr TileRule f32_tile_rule() { return {2560, false}; }
+
+// lines per tile: the largest power of two (at most `most` lines) that the rule allows
+__host__ __device__ inline int tile_lines_log2(const FftPlan& p, TileRule r, int most) {
     int ln = 0;
     const int nb = p.nst ? p.L / p.radix[0] : 1;
-    while ((2 << ln) <= 32 && (1 << ln) < most && (p.L << (ln + 1)) <= points && (!dd || (nb << (ln + 1)) <= 256)) ++ln;
+    while ((2 << ln) <= 32 && (1 << ln) < most && (p.L << (ln + 1)) <= r.points &&
+           (!r.one_round || (nb << (ln + 1)) <= 256))
+        ++ln;
     return ln;
 }
 __host__ __device__ inline int tile_threads(const FftPlan& p, int ln) {
@@ -60,8 +71,6 @@ __host__ __device__ inline int tile_threads(const FftPlan& p, int ln) {
     const int t = ((((p.L / r) << ln) + 31) / 32) * 32;
     return t < 64 ? 64 : (t > 256 ? 256 : t);
 }
-
-constexpr int kDdTilePoints = 1700, kF32TilePoints = 2560;
 
 // values of a transform: memory type, twiddles in the plan's stage order, arithmetic
 template <typename V>
