@@ -982,13 +982,18 @@ mvd_status mvd_precompute_kernels(mvd_ctx* c, int variant) {
     if (variant == MVD_EFFICIENT)
         MVD_TRY(autocorr_all(c->nv, c->d_psf, c->koff.data(), c->kd.data(), c->d_ktmp, (long)qmax, c->stream));
     MVD_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), c->stream));
-    float* factors = nullptr;  // of the views built at once: given back before the engine takes its buffers
-    if (nc) MVD_TRY(dev_alloc(&factors, nc, "compound factors"));
+    // the factors of the views built at once: in the ratio buffer, else in one of their own, which
+    // is given back before the engine takes its spectra
+    float *own = nullptr, *factors = c->d_r;
+    if (nc > (size_t)c->M) {
+        MVD_TRY(dev_alloc(&own, nc, "compound factors"));
+        factors = own;
+    }
     int bad = 0;
     mvd_status built = build_compounds(c->nv, c->d_psf, c->koff.data(), c->kd.data(), variant, c->d_comp, c->d_ktmp,
                                        (long)qmax, factors, group, c->d_flag, c->stream);
     if (built == MVD_OK) built = read_flag(c, &bad);
-    dev_free(factors);
+    dev_free(own);
     MVD_TRY(built);
     if (bad) {
         set_error("mvd_precompute_kernels: a compound kernel sums to zero");
