@@ -184,12 +184,16 @@ __host__ __device__ __forceinline__ cdp cdp_two_sub(cdp x, cdp y) {
     const f2 e = f2_add(f2_sub(x.h, f2_add(s, nb)), f2_sub(nb, y.h));
     return {s, f2_add(e, f2_sub(x.l, y.l))};
 }
+// x plus y with its parts exchanged and multiplied by the signs s (exact)
+__host__ __device__ __forceinline__ cdp cdp_two_addx(cdp x, cdp y, f2 s) {
+    const f2 yh = f2_swap(y.h);
+    const f2 t = f2_fma(yh, s, x.h), nb = f2_sub(x.h, t);
+    const f2 e = f2_add(f2_sub(x.h, f2_add(t, nb)), f2_fma(yh, s, nb));
+    return {t, f2_add(e, f2_fma(f2_swap(y.l), s, x.l))};
+}
 template <int S>
 __host__ __device__ __forceinline__ cdp cdp_two_addi(cdp x, cdp y) {
-    const f2 i = f2_si<S>(), yh = f2_swap(y.h);
-    const f2 s = f2_fma(yh, i, x.h), nb = f2_sub(x.h, s);
-    const f2 e = f2_add(f2_sub(x.h, f2_add(s, nb)), f2_fma(yh, i, nb));
-    return {s, f2_add(e, f2_fma(f2_swap(y.l), i, x.l))};
+    return cdp_two_addx(x, y, f2_si<S>());
 }
 // x y as an unevaluated pair (dd_dot2_pair): 16 instructions
 __host__ __device__ __forceinline__ cdp cdp_mul_pair(cdp x, cdp y) {

@@ -356,7 +356,10 @@ __device__ __forceinline__ void unpack_pair(float2 zk, float2 zm, float2& a, flo
 }
 // and back: the full spectrum of a + i b at k (up: k <= L/2) or at L - k
 __device__ __forceinline__ cdp pack_pair(cdp a, cdp b, bool up) {
-    return up ? cdp_two_addi<+1>(a, b) : cdp_conj(cdp_two_addi<-1>(a, b));
+    // up: a + i b; else conj(a - i b) = conj(a) + i conj(b)
+    const f2 c = up ? 0ull : 0x8000000000000000ull;
+    a.h ^= c, a.l ^= c;
+    return cdp_two_addx(a, b, up ? f2_of(-1.f, 1.f) : f2_of(1.f, 1.f));
 }
 __device__ __forceinline__ float2 pack_pair(float2 a, float2 b, bool up) {
     return up ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, b.x - a.y);
