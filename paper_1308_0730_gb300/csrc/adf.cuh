@@ -1,6 +1,8 @@
 // Aligned double-float: the arithmetic of the double-float FFT lines, in scalar
-// form (also compiled for the host). The passes run the same operations on packed
-// FP32 pairs (adp.cuh), with the same roundings.
+// form. The passes run the same operations, with the same roundings, on packed FP32
+// pairs (adp.cuh, which a host check compiles too: tests/native/line_host_check.cu) and
+// take only the grid functions from here; the scalar values and butterflies are the form
+// that tests/native/adf_host_check.cu compiles for the host.
 //
 // A value is the unevaluated sum hi + lo of two FP32 numbers, as in dd.cuh,
 // with one more invariant: every hi of a line is an integer multiple of the
@@ -22,7 +24,8 @@
 // 9.7 times that, and the next stage's twiddle product to 13.7 times; the next
 // stage therefore runs at quantum 16 q, where the bound is again 2^19. The
 // magic-constant rounding needs |x| <= 2^22 q and the butterfly's sums stay
-// below 2^23 q.
+// below 2^23 q. Radix-16 stages start from 2^18 q and move to 32 q; mixed-radix lines
+// run their first stage without a grid (adf_second_exp, adf_gen_shift below).
 //
 // Every operation uses the _rn intrinsics, which the compiler neither
 // contracts into FMAs nor reassociates.

@@ -2,7 +2,9 @@
 // register pairs, the high parts (re, im) and the low parts (re, im), and every
 // operation is one two-lane FP32 instruction (add/mul/fma.rn.f32x2, each lane
 // rounded as its scalar form). The steps are those of adf.cuh, operation for
-// operation, so the results are bit-identical to it.
+// operation, so the results are bit-identical to it. The same
+// butterflies also run without a grid (Unaligned: TwoSum sums, renormalised products), as
+// the first stage of a mixed-radix line does.
 //
 // Why: the FFT passes are bound by issue slots and shared memory, not by the FP32
 // lanes. One radix-8 stage with its twiddles takes 23 instructions per point

@@ -20,7 +20,7 @@
 //     asynchronous copies (all in flight at once), two or more blocks per SM
 //     overlapping one's copies with another's sums.
 // Measured against one output row per thread with scalar loads (GB300, one launch,
-// us): 32^3 outputs, 13x7x7 box 52.9 -> 8.3; 97x83x61, 9x9x15 222 -> 45;
+// us): 32^3 outputs, 13x7x7 box 52.9 -> 8.3; 97x83x61, 9x9x15 222 -> 44;
 // 120x110x100, 15x15x41 about 0.46 of the FMA peak (660 us).
 // The order of each output's sum in the direct engine depends on S only (and, where not one
 // row of taps fits, on the pieces): not on NY, CK, the warps or the rows staged at a time,

@@ -76,7 +76,7 @@ cudaError_t allow_smem(K kern) {
 // last block of the stream's previous kernel exits, without waiting for that kernel's
 // completion to reach the front end, and its blocks wait (pass_wait) for it before they
 // touch memory. Every kernel launched this way calls pass_wait first. Measured: a
-// calibration step on 128x128x96 (about 900 launches of 6-20 us) 25.8 -> 21.9 ms, ten
+// calibration step on 128x128x96 (about 900 launches of 6-20 us) 25.8 -> 21.5 ms, ten
 // iterations of 32^3 556 -> 491 us; letting the next grid start with the running one's
 // first instruction instead (its waiting blocks then hold registers and shared memory) 23.5
 // ms and 534 us.

@@ -6,9 +6,11 @@ namespace mvd {
 
 namespace {
 
-// Mixed-radix double-float passes: four blocks of 256 threads per SM (64 registers; a
-// few bytes of spills). They wait on loads more than they issue: 300x180x150, a view
-// update with 3, 4 and 5 blocks (the tiles sized to fit) 739, 661 and 698 us.
+// Mixed-radix double-float passes: four blocks of 256 threads per SM. At 64 registers they
+// spill (bytes stored and loaded: z with the product 188 and 332, update 112 and 328, ratio
+// 124 and 244, the others at most 76 and 112), but they wait on loads more than they issue:
+// 300x180x150, a view update with 3, 4 and 5 blocks (the tiles sized to fit, all passes
+// together) 739, 661 and 698 us.
 constexpr int kDdGenBlocks = 4;
 
 __global__ void __launch_bounds__(kGenThreads, kDdGenBlocks) k_dd_x_forward(const __grid_constant__ DdX a) {

@@ -16,14 +16,15 @@
 //     the bound of the first stage's outputs gives. Aligning the inputs instead, with the
 //     worst growth of every stage assumed, costs 1.5 bits in the mean and 3 on lines with
 //     spikes (errors against 80-bit transforms, tests/native/line_host_check.cu), and was
-//     no faster (300x180x150, a view update: 584 us; now 583);
+//     no faster: a view update of 300x180x150 584 us, now 582, 288x288x144 754 and 729,
+//     90x60x48 100 and 98, but 200x96x100 200 and 212;
 //   - tiles of up to 1700 points (54 KB with both exchange buffers) and blocks of as
 //     many threads as the second stage has butterflies: four or more per SM; operands
 //     that only the last stage reads are prefetched into L2 when the block starts.
 //
-// Measured on 300x180x150 (us a launch, before -> now): x forward 100 -> 50, y 65 -> 40,
-// z 135 -> 92, ratio 207 -> 112, update 158 -> 76; instructions per point of the y pass
-// 342 -> 180. Loads in flight bound them still (a third of the warps resident).
+// Measured on 300x180x150 (us a launch, against passes that load, transform and store one
+// after another): x forward 100 -> 51, y 65 -> 39, z 135 -> 90, ratio 207 -> 116, update
+// 158 -> 81. Loads in flight bound them still (a third of the warps resident).
 #pragma once
 
 #include "adf.cuh"
