@@ -134,8 +134,11 @@ inline bool bc_plan(int ox, int oy, int oz, int kx, int ky, int kz, int ny_max, 
                 if (bc_plan_ny(ox, oy, oz, kx, ky, kz, ny, s, warps, &p) && (!any || p.cost < best->cost))
                     *best = p, any = true;
             }
-    return any || bc_plan_ny(ox, oy, oz, kx, ky, kz, 1, bc_splits((long)((ox + 31) / 32) * ((oy + 7) / 8) * oz, kz), 8,
-                             best, true);
+    if (any) return true;
+    const int s = bc_splits((long)((ox + 31) / 32) * ((oy + 7) / 8) * oz, kz);
+    if (!bc_plan_ny(ox, oy, oz, kx, ky, kz, 1, s, 8, best, true)) return false;
+    best->ck = 1;  // a chain runs on over the stagings of one plane
+    return true;
 }
 
 // A batch of convolutions of small kernels (zero outside their boxes), one

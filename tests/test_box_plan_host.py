@@ -72,7 +72,8 @@ def test_tile_choice_does_not_change_the_order_of_sums(plan):
     """Splits of the tap planes and pieces of their rows: the same for ty = 8 and ty = 4. (The rows
     staged at a time may differ: their chains run on, tests/test_gpu_direct_heights.py.)"""
     rng = random.Random(5)
-    cases = [((200, 80, 40), (101, 41, 3)), ((194, 356, 87), (1, 191, 3)), ((40, 194, 78), (11, 95, 1))]
+    cases = [((200, 80, 40), (101, 41, 3)), ((194, 356, 87), (1, 191, 3)), ((40, 194, 78), (11, 95, 1)),
+             ((6600, 1, 1), (6501, 1, 1)), ((7000, 3, 9), (6501, 1, 5)), ((7000, 9, 9), (6501, 3, 3))]  # in pieces
     while len(cases) < 4000:
         box = tuple(2 * rng.randrange(0, int(10 ** rng.uniform(0.3, 2.0))) + 1 for _ in range(3))
         if accepted(*box):
