@@ -247,7 +247,7 @@ __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz
     const int lx = lane & 3, ly = lane >> 2;
     const int nw = blockDim.x >> 5, nz = nw / S, s = warp & (S - 1), zl = warp / S;
     const int x0 = bx * kBcTX, y0 = by * 8 * NY, z0 = bz * nz;
-    constexpr bool PIECES = KX < 0, ROWS = PIECES || COMP, CHAIN = PIECES && !COMP;
+    constexpr bool PIECES = KX < 0, CHAIN = PIECES && !COMP;
     const int px = PIECES ? j.cx : j.kx;
     const int wx = bc_wx(px), kxp = bc_kxp(px);
     int nf = px >> 2, rem = px & 3;
@@ -275,9 +275,9 @@ __device__ __forceinline__ void bc_tile(const BoxConv& j, int bx, int by, int bz
 #pragma unroll
         for (int i = 0; i < 8; ++i) tot[o][i] = 0.f, cmp[o][i] = 0.f;
     for (int k0 = klo; k0 < khi; k0 += j.ck)
-        for (int q0 = 0; q0 < (ROWS ? j.ky : 1); q0 += ROWS ? j.cy : 1)
+        for (int q0 = 0; q0 < j.ky; q0 += j.cy)
             for (p0 = 0; p0 < (PIECES ? j.kx : 1); p0 += PIECES ? j.cx : 1) {
-                const int ck = min(j.ck, khi - k0), cy = ROWS ? min(j.cy, j.ky - q0) : j.ky;
+                const int ck = min(j.ck, khi - k0), cy = min(j.cy, j.ky - q0);
                 const int nx = PIECES ? min(j.cx, j.kx - p0) : j.kx;  // taps of the piece's rows
                 if constexpr (PIECES) {
                     gxa = column(lane, oka), gxb = column(lane + 32, okb);

@@ -38,33 +38,45 @@ struct DArgs {
 enum { M_RATIO, M_UPDATE, M_CONV, M_ADD, M_ACCUMULATE };
 
 // M_RATIO: out = phi / max(conv, eps); M_UPDATE: out = max(out . conv, eps); M_CONV: out = conv;
-// M_ADD: out += conv; M_ACCUMULATE: out *= conv (the combined update's product). KX: the box's
-// length in x, 0 for those without a kernel of their own, -1 for planes staged in rows.
-// Blocks of 256 threads have 80 registers, for three of them per SM: with one kernel for both
-// sizes of block the 8-row tiles took 82 to 103, which left two (97x83x61, 9x9x15: 48.4 against
-// 44.7 us a launch); held to 80, blocks of 512 gain nothing (three updates of 32^3: 69 and 73 us).
+// M_ADD: out += conv; M_ACCUMULATE: out *= conv (the combined update's product).
+__device__ __forceinline__ void finish(const DArgs& a, long g, float acc) {
+    if (a.mode == M_RATIO) {
+        a.out[g] = __ldg(a.phi + g) / fmaxf(acc, a.eps);
+    } else if (a.mode == M_UPDATE) {
+        const float p = a.out[g];
+        a.out[g] = fmaxf(p * (a.wt || a.lam != 0.f || a.inv_s ? update_factor(acc - 1.f, p, a.wt, g, a.lam, a.inv_s)
+                                                              : acc),
+                         a.eps);
+    } else if (a.mode == M_CONV) {
+        a.out[g] = acc;
+    } else if (a.mode == M_ADD) {
+        a.out[g] += acc;
+    } else {
+        a.out[g] *= a.inv_s ? acc * __ldg(a.inv_s + g) : acc;
+    }
+}
+
+// KX: the box's length in x, 0 for those without a kernel of their own, -1 for planes staged in
+// rows. Blocks of 256 threads have 80 registers, for three of them per SM: with one kernel for
+// both sizes of block the 8-row tiles took 82 to 103, which left two (97x83x61, 9x9x15: 48.4
+// against 44.7 us a launch); held to 80, blocks of 512 gain nothing (three updates of 32^3: 69
+// and 73 us).
 template <int NY, int KX, int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 1) k_direct(const __grid_constant__ DArgs a) {
     extern __shared__ float4 smem4[];
     pass_wait();
     bc_tile<NY, KX, true, false>(a.c, blockIdx.x, blockIdx.y, blockIdx.z, a.splits, reinterpret_cast<float*>(smem4),
                                  [&](int x, int y, int z, float acc) {
-        const long g = (long)x + (long)a.c.ox * (y + (long)a.c.oy * z);
-        if (a.mode == M_RATIO) {
-            a.out[g] = __ldg(a.phi + g) / fmaxf(acc, a.eps);
-        } else if (a.mode == M_UPDATE) {
-            const float p = a.out[g];
-            a.out[g] = fmaxf(p * (a.wt || a.lam != 0.f || a.inv_s ? update_factor(acc - 1.f, p, a.wt, g, a.lam, a.inv_s)
-                                                                  : acc),
-                             a.eps);
-        } else if (a.mode == M_CONV) {
-            a.out[g] = acc;
-        } else if (a.mode == M_ADD) {
-            a.out[g] += acc;
-        } else {
-            a.out[g] *= a.inv_s ? acc * __ldg(a.inv_s + g) : acc;
-        }
+        finish(a, (long)x + (long)a.c.ox * (y + (long)a.c.oy * z), acc);
     });
+}
+
+// One tap: nothing to stage, memory bound (two views of 128^3: 82 us an iteration through the
+// tiles, 72 with one output row per thread; 27 here; 32^3 23, 19 and 8.7).
+__global__ void __launch_bounds__(256) k_point(const __grid_constant__ DArgs a, long n) {
+    pass_wait();
+    const float t = __ldg(a.c.taps);
+    for (long g = blockIdx.x * 256L + threadIdx.x; g < n; g += 256L * gridDim.x) finish(a, g, t * a.c.in[g]);
 }
 
 template <int NY, int THREADS>
@@ -103,10 +115,14 @@ mvd_status launch(DArgs& a, int mode, cudaStream_t st, const char* name, int ty 
     if (e != cudaSuccess) return cuda_status(e, name);
     const int nz = p.planes();
     const dim3 grid((c.ox + kBcTX - 1) / kBcTX, (c.oy + 8 * p.ny - 1) / (8 * p.ny), (c.oz + nz - 1) / nz);
+    const long n = (long)c.ox * c.oy * c.oz, points = (n + 255) / 256;
     const int cls = mode == M_RATIO ? KC_DIRECT_RATIO
                                     : (mode == M_UPDATE || mode == M_ACCUMULATE) ? KC_DIRECT_UPDATE : KC_DIRECT_CONV;
     prof_begin(cls, st);
-    e = launch_pass(kern, grid, 32 * p.warps, p.smem, st, a);
+    if (c.kx * c.ky * c.kz == 1)
+        e = launch_pass(k_point, dim3((unsigned)(points < 152 * 16 ? points : 152 * 16)), 256, 0, st, a, n);
+    else
+        e = launch_pass(kern, grid, 32 * p.warps, p.smem, st, a);
     prof_end(cls, st);
     if (e != cudaSuccess) return cuda_status(e, name);
     count_launch();
