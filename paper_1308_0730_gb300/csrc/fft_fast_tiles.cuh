@@ -135,15 +135,25 @@ __device__ __forceinline__ void x_load_packed(const XFast& a, float2 (&v)[kE], f
     constexpr int TPL = L / kE, P = kFastThreads / TPL, XH = L / 2 + 1;
     static_assert(2 * P * XH <= P * line_stride(L), "the gathered rows exceed the lines' buffer");
     const float2* spec = a.spec + rho0;
-    for (int idx = threadIdx.x; idx < XH * 2 * P; idx += kFastThreads) {
-        const int k = idx / (2 * P), row = idx - k * 2 * P;
-        const bool ok = row < nrows;
-        if constexpr (CO)  // an 8-byte asynchronous copy would go through L1
-            sm[row * XH + k] = ok ? ld2<CO>(spec + (long)k * a.YZ + row) : make_float2(0.f, 0.f);
-        else
+    if constexpr (CO) {  // an 8-byte asynchronous copy would go through L1: all loads before the first store
+        constexpr int KS = kFastThreads / (2 * P), N = (XH + KS - 1) / KS;  // k of a thread's elements: KS apart
+        static_assert(KS >= 1, "a tile has more rows than threads");
+        const int row = threadIdx.x % (2 * P), k0 = threadIdx.x / (2 * P);
+        float2 t[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            t[j] = row < nrows && k0 + j * KS < XH ? ld2<CO>(spec + (long)(k0 + j * KS) * a.YZ + row) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (k0 + j * KS < XH) sm[row * XH + k0 + j * KS] = t[j];
+    } else {
+        for (int idx = threadIdx.x; idx < XH * 2 * P; idx += kFastThreads) {
+            const int k = idx / (2 * P), row = idx - k * 2 * P;
+            const bool ok = row < nrows;
             cp_async8(sm + row * XH + k, ok ? spec + (long)k * a.YZ + row : a.spec, ok);
+        }
+        cp_async_wait_all();
     }
-    cp_async_wait_all();
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kE; ++q) {
@@ -185,20 +195,29 @@ __device__ __forceinline__ void fast_x_inverse_tile(const XFast& a, long tile, f
     const int nrows = (int)min((long)2 * P, a.YZ - rho0);
     const bool oka = p < nrows, okb = P + p < nrows;
     // the epilogue's operand rows (phi for the ratio, psi for the update) come into L2
-    // meanwhile: loaded here they would hold 32 registers through the transform
-    if (MODE == 0) prefetch_rows(a.phi + rho0 * L, nrows * L * 4);
-    if (MODE == 1 || MODE == 4) prefetch_rows(a.psi + rho0 * L, nrows * L * 4);
+    // meanwhile: loaded here they would hold 32 registers through the transform. The persistent
+    // batch kernel (CO: two blocks, 128 registers) has those, and hides less: four volumes of
+    // 128^3 in FP32 1.48 ms with prefetches and one gathered value at a time, 1.27 so.
+    if (!CO && MODE == 0) prefetch_rows(a.phi + rho0 * L, nrows * L * 4);
+    if (!CO && (MODE == 1 || MODE == 4)) prefetch_rows(a.psi + rho0 * L, nrows * L * 4);
     float2 v[kE];
     x_load_packed<L, CO>(a, v, sm, p, t, rho0, nrows);
     const long ra = (rho0 + p) * L, rb = (rho0 + P + p) * L;
-    LineFFT<L, +1, true>::run(v, sm + p * LS, t, a.tw);
-    if (MODE == 0) {
-        float2 w[kE];  // all loads before the first division (whose slow path is a branch)
+    float2 w[kE];
+    auto operands = [&] {
 #pragma unroll
         for (int q = 0; q < kE; ++q) {
             const int n = t + TPL * q;
-            w[q] = make_float2(oka ? __ldg(a.phi + ra + n) : 0.f, okb ? __ldg(a.phi + rb + n) : 0.f);
+            if (MODE == 0)
+                w[q] = make_float2(oka ? __ldg(a.phi + ra + n) : 0.f, okb ? __ldg(a.phi + rb + n) : 0.f);
+            else
+                w[q] = make_float2(oka ? ld1<CO>(a.psi + ra + n) : 0.f, okb ? ld1<CO>(a.psi + rb + n) : 0.f);
         }
+    };
+    if (CO && MODE != 2) operands();
+    LineFFT<L, +1, true>::run(v, sm + p * LS, t, a.tw);
+    if (MODE == 0) {
+        if (!CO) operands();  // all loads before the first division (whose slow path is a branch)
 #pragma unroll
         for (int q = 0; q < kE; ++q) {
             // r - 1 (see the generic ratio pass): the update adds the 1 back
@@ -214,7 +233,8 @@ __device__ __forceinline__ void fast_x_inverse_tile(const XFast& a, long tile, f
             const int n = t + TPL * q;
             if (MODE == 1) {
                 // v = c - 1 (weights and regularisation: update_factor)
-                const float pa = oka ? ld1<CO>(a.psi + ra + n) : 0.f, pb = okb ? ld1<CO>(a.psi + rb + n) : 0.f;
+                const float pa = CO ? w[q].x : oka ? ld1<CO>(a.psi + ra + n) : 0.f;
+                const float pb = CO ? w[q].y : okb ? ld1<CO>(a.psi + rb + n) : 0.f;
                 if (oka) a.psi[ra + n] = fmaxf(pa * update_factor(v[q].x, pa, a.wt, ra + n, a.lam, a.inv_s), a.eps);
                 if (okb) a.psi[rb + n] = fmaxf(pb * update_factor(v[q].y, pb, a.wt, rb + n, a.lam, a.inv_s), a.eps);
             } else if (MODE == 4) {  // combined update: multiply this view's factor into the product

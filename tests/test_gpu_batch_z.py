@@ -49,3 +49,32 @@ def test_register_resident_axes(specs):
         if g.size < 200000:
             want, _ = oracle.deconvolve(w.views, w.psfs, 2, "efficient")
             assert rel_err(g, want) < PARITY_TOL, f"{w.name}: {err_report(g, want)}"
+
+
+@pytest.mark.parametrize("dims", [(64, 12, 9), (128, 10, 9), (256, 9, 8), (128, 64, 64), (64, 33, 10)])
+def test_fp32_x_tiles(dims):
+    """FP32 persistent runs on register-resident x lengths: full tiles and tiles with rows past the end."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import numpy as np
+
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_1308_0730_gb300 import mvd
+
+    dims = tuple(synth.workloads.smooth235(n) for n in dims)
+    w = synth.small_case(950, dims=dims, n_views=2, n_iter=2, asymmetric=True)
+    # a constant background keeps b away from the floor, where FP32 transforms lose the bar
+    views = [v + np.float32(20) for v in w.views]
+    want, _ = oracle.deconvolve(views, w.psfs, 2, "efficient")
+    with mvd.Deconvolver(views, w.psfs, "efficient", path="fft", precision="fast", stream=torch.cuda.Stream()) as d:
+        b = mvd.mvd_batch_create([d], 2, "persistent")
+        try:
+            mvd.mvd_batch_run(b)
+            mvd.mvd_batch_wait(b)
+            got = d.result()
+        finally:
+            mvd.mvd_batch_destroy(b)
+    assert rel_err(got, want) < PARITY_TOL, err_report(got, want)
